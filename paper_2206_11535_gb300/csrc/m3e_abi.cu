@@ -125,7 +125,7 @@ struct m3e_ctx {
   StreamEngine* stream = nullptr;
   // fit gradient: per-block partial sums and the valid-candidate counter
   double* fit_partial = nullptr;
-  int fit_partial_blocks = 0;
+  int fit_bpsm = 1, fit_grad_bpsm = 1;
   unsigned long long* fit_nvalid = nullptr;
   unsigned long long* h_fit_nvalid = nullptr;
 };
@@ -458,6 +458,8 @@ int m3e_create(const m3e_config* cfg, int cuda_device, m3e_ctx** out) {
   x->s1c_bpsm = stage_blocks_per_sm(5);
   x->s1m_bpsm = stage_blocks_per_sm(6);
   x->ingest_bpsm = ingest_blocks_per_sm();
+  x->fit_bpsm = fit_grad_blocks_per_sm(false);
+  x->fit_grad_bpsm = fit_grad_blocks_per_sm(true);
   // look-up tables in FP64, rounded once
   int ncolt = 0, nrowt = 0;
   for (int L = 0; L < 4; ++L) {
@@ -1149,16 +1151,12 @@ int fit_call(m3e_ctx* x, const int32_t* d_hits, const int64_t* d_off, int64_t n_
     return fail(M3E_EINVAL, "frame_off, params, cand and hits must not be NULL");
   if (((uintptr_t)d_cand & 15) != 0) return fail(M3E_EINVAL, "cand must be 16-byte aligned (rows of 4 int32)");
   DeviceGuard guard(x->device);
-  const int nb = fit_grad_blocks(x->sms, n_cand);
-  if (nb > x->fit_partial_blocks) {
-    cudaFree(x->fit_partial);
-    x->fit_partial = nullptr;
-    x->fit_partial_blocks = 0;
-    CUDA_TRY(cudaMalloc(&x->fit_partial, sizeof(double) * fit_grad_partial_size() * (size_t)nb));
-    x->fit_partial_blocks = nb;
+  if (!x->fit_partial) {  // one slot per block of the larger grid
+    const size_t slots = (size_t)x->sms * std::max(x->fit_bpsm, x->fit_grad_bpsm);
+    CUDA_TRY(cudaMalloc(&x->fit_partial, sizeof(double) * fit_grad_partial_size() * slots));
   }
+  const int nb = fit_grad_blocks(x->sms * (grad ? x->fit_grad_bpsm : x->fit_bpsm), n_cand);
   if (!x->fit_nvalid) CUDA_TRY(cudaMalloc(&x->fit_nvalid, sizeof(unsigned long long)));
-  CUDA_TRY(cudaMemsetAsync(x->fit_nvalid, 0, sizeof(unsigned long long), s));
   CUDA_TRY(launch_fit_grad(x->dc, d_hits, d_off, n_frames, d_cand, n_cand, d_params, x->col_lut, x->row_lut,
                            x->fit_partial, nb, x->fit_nvalid, chi2_each, kappa_each, chi2_sum, grad, s));
   return M3E_OK;

@@ -258,25 +258,6 @@ __device__ __forceinline__ SegF segment_core(float d, float z, float Rct, float 
   return s;
 }
 
-// The same from the chord alone: sin(Phi/2) = d / 2R_t on either arc (the long arc
-// turns by 2 pi minus the short one, which leaves the sine of the half angle and
-// flips its cosine); inv2R = 1 / (2 R_t).  Near a half turn (d -> 2 R_t) the arc
-// sine loses half the digits of its argument; the triplet fit therefore takes the
-// angle from the triangle (fit_triplet), and this form serves the reverse sweep of
-// the alignment gradient, which differentiates it.
-__device__ __forceinline__ SegF segment(float d, float z, float Rct, float inv2R, bool obtuse) {
-  const float sh = fminf(1.f, d * inv2R);
-  float ph = 2.f * asinf(sh);
-  float ch = sqrtf(fmaxf((1.f - sh) * (1.f + sh), 0.f));
-  if (obtuse) {
-    ph = TWO_PI_F - ph;
-    ch = -ch;
-  }
-  SegF s = segment_core(d, z, Rct, sh, ch, ph);
-  s.th = atan2f(Rct * ph, z);
-  return s;
-}
-
 struct TFitF {
   float eps, Rct, ccx, ccy;
   float Rref;                  // expansion point of the kink model: R_C of segment 0
@@ -285,6 +266,7 @@ struct TFitF {
   float kappa, skappa;
   float zp0, RC0, dth0;         // segment 0: z / Phi (theta_C0 = atan2(Rct, zp0)), R_C, dtheta/dR
   float zp1;                   // z / Phi of segment 1 = R_t cot(theta_C1)
+  float ph0, ph1;              // arc angles of the segments (alignment gradient)
   int valid;
 };
 
@@ -324,8 +306,10 @@ __device__ __forceinline__ TFitF fit_triplet(float ax, float ay, float az, float
   const float dotc = (ax - cx) * (bx - cx) + (ay - cy) * (by - cy);
   const float dota = (bx - ax) * (cx - ax) + (by - ay) * (cy - ay);
   const float il0 = 1.f / (d20 * d12), il1 = 1.f / (d01 * d20);
-  const SegF s0 = segment_core(d01, bz - az, f.Rct, acr * il0, dotc * il0, 2.f * atan2f(acr, dotc));
-  const SegF s1 = segment_core(d12, cz - bz, f.Rct, acr * il1, dota * il1, 2.f * atan2f(acr, dota));
+  f.ph0 = 2.f * atan2f(acr, dotc);
+  f.ph1 = 2.f * atan2f(acr, dota);
+  const SegF s0 = segment_core(d01, bz - az, f.Rct, acr * il0, dotc * il0, f.ph0);
+  const SegF s1 = segment_core(d12, cz - bz, f.Rct, acr * il1, dota * il1, f.ph1);
   const float dR = s0.RC - s1.RC;
   f.Rref = s0.RC;
   f.alpha = 0.5f * (s0.dphi + s1.dphi);
@@ -413,7 +397,7 @@ __device__ __forceinline__ TFitF unpark_fit(const FitPark& pk) {
   f.zp0 = q[9 * 128];
   f.dth0 = q[10 * 128];
   f.RC0 = f.Rref;  // R_C of segment 0 is the expansion point
-  f.eps = f.ccx = f.ccy = f.zp1 = 0.f;
+  f.eps = f.ccx = f.ccy = f.zp1 = f.ph0 = f.ph1 = 0.f;
   f.valid = 1;
   return f;
 }

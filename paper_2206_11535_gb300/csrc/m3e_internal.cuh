@@ -127,7 +127,8 @@ cudaError_t launch_ingest(const DevCfg& c, const int32_t* hits, int64_t n, const
                           float* x, float* y, float* z, float* phi, int* err, int grid, cudaStream_t s);
 
 // Gradient of the fit chi2 (m3e_grad.cu).
-int fit_grad_blocks(int sms, int64_t n_cand);
+int fit_grad_blocks_per_sm(bool grad);
+int fit_grad_blocks(int resident, int64_t n_cand);
 int fit_grad_partial_size();
 cudaError_t launch_fit_grad(const DevCfg& c, const int32_t* hits, const int64_t* off, int64_t n_frames,
                             const int32_t* cand, int64_t n_cand, const float* params, const float4* col_lut,
