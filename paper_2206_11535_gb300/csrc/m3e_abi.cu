@@ -268,15 +268,27 @@ int grow(T*& ptr, int64_t& cap, int64_t need, size_t elem, const char* what) {
   return M3E_OK;
 }
 
-// Scratch for a batch of nf frames (staged arrays only when staged; the sorted
-// hits of pending frames take HITS_PER_FRAME entries per frame on average, frames
-// beyond that are deferred to the CTA-per-frame kernel).
-constexpr int64_t HITS_PER_FRAME = 128;
+// Scratch for a batch of nf frames (staged arrays only when staged).  The sorted hits,
+// triplets and combinations of a batch share its scratch, and frames that find it full go
+// to the CTA-per-frame kernel, which runs them many times slower.  The sizes per frame are
+// those of the throughput mix (85 hits, 44 triplets) with a margin; a batch of denser
+// frames needs more, so up to the scratch of ROOMY_FRAMES frames a batch gets the second,
+// roomier figure (20,001 frames of 32 tracks, 137 hits and 108 triplets each: 7,000 frames
+// deferred and 855 us with the first figures alone).
+constexpr int64_t ROOMY_FRAMES = 1 << 20;
+constexpr int64_t HITS_PER_FRAME[2] = {128, 512};
+constexpr int64_t TRIPLETS_PER_FRAME[2] = {64, 512};
+constexpr int64_t COMBOS_PER_FRAME[2] = {192, 384};
+
+int64_t scratch_entries(const int64_t (&per_frame)[2], int64_t nf) {
+  // indices travel as int32 in the records: at most 2^31 - 2^16 entries
+  const int64_t lim = ((int64_t)1 << 31) - (1 << 16);
+  const int64_t roomy = std::min(per_frame[1] * nf, per_frame[0] * ROOMY_FRAMES);
+  return std::min(std::max({per_frame[0] * nf, roomy, (int64_t)1 << 16}), lim);
+}
 
 int ensure_scratch(Scratch& sc, int64_t nf, bool staged) {
-  // sorted-hit indices travel as int32 in the triplet records: at most 2^31 - 2^16 of them
-  const int64_t nh_want = nf * HITS_PER_FRAME > (1 << 16) ? nf * HITS_PER_FRAME : (1 << 16);
-  const int64_t nh = nh_want < ((int64_t)1 << 31) - (1 << 16) ? nh_want : ((int64_t)1 << 31) - (1 << 16);
+  const int64_t nh = scratch_entries(HITS_PER_FRAME, nf);
   int64_t one = sc.work ? 1 : 0;
   int rc = grow(sc.work, one, 1, 4 * sizeof(int), "work counters");
   if (rc) return rc;
@@ -312,9 +324,7 @@ int ensure_scratch(Scratch& sc, int64_t nf, bool staged) {
     if (rc) return rc;
     sc.frames_cap = nf;
   }
-  const int64_t lim = ((int64_t)1 << 31) - (1 << 16);
-  int64_t tc = 64 * nf > (1 << 16) ? 64 * nf : (1 << 16);
-  tc = tc < lim ? tc : lim;
+  const int64_t tc = scratch_entries(TRIPLETS_PER_FRAME, nf);
   if (tc > sc.trip_cap) {
     int64_t c0 = sc.trip_cap, c1 = sc.trip_cap, c2 = sc.trip_cap;
     rc = grow(sc.trip, c0, tc, sizeof(int4), "triplets");
@@ -323,8 +333,7 @@ int ensure_scratch(Scratch& sc, int64_t nf, bool staged) {
     if (rc) return rc;
     sc.trip_cap = tc;
   }
-  int64_t cc = 192 * nf > (1 << 16) ? 192 * nf : (1 << 16);
-  cc = cc < lim ? cc : lim;
+  const int64_t cc = scratch_entries(COMBOS_PER_FRAME, nf);
   return grow(sc.combo, sc.combo_cap, cc, sizeof(int4), "combinations");
 }
 
