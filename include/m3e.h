@@ -151,8 +151,10 @@ int m3e_destroy(m3e_ctx* ctx);
  * the throughput form: five persistent kernels that regroup the batch by
  * candidate (frames -> selected triplets -> tracks -> combinations -> decisions,
  * the candidates in device scratch); frames larger than a stage's capacity are
- * re-run by a CTA-per-frame kernel with identical decisions.  d_stats may be
- * NULL.  n_frames may be 0. */
+ * re-run by a CTA-per-frame kernel with identical decisions.  A batch of at most
+ * 2048 frames without statistics or kernel timing runs a CTA per frame instead
+ * (two launches, no scratch, the same decisions).  d_stats may be NULL.  n_frames
+ * may be 0. */
 int m3e_select_frames(m3e_ctx* ctx, const int32_t* d_hits, const int64_t* d_frame_off, int64_t n_frames,
                       uint8_t* d_keep, uint8_t* d_reason, m3e_stats* d_stats, cudaStream_t stream);
 
@@ -286,7 +288,8 @@ int m3e_ingest(m3e_ctx* ctx, const int32_t* d_hits, int64_t n_hits, float* d_x, 
  * device synchronisation of cudaMalloc/cudaFree, and a process sharing the GPU
  * under a fixed memory budget reserves all memory at start-up.  The context must
  * exist already (m3e_create allocates; create it during initialisation).
- *   - At most 262,144 frames per call; more returns M3E_EINVAL.
+ *   - At most 262,144 frames per call; more returns M3E_EINVAL.  At most 2048
+ *     frames run a CTA per frame and do not touch the array.
  *   - The first call on a device looks up the array's device address (set-up);
  *     make that first call before any stream capture.  The address is cached per
  *     device; m3e_create clears the cache, so after a cudaDeviceReset create a

@@ -393,11 +393,27 @@ int check_batch(const int32_t* hits, const int64_t* off, int64_t n, const uint8_
 
 enum { FORM_STAGED = 0, FORM_FUSED = 1, FORM_PLAIN = 2 };
 
-// Enqueue one batch on stream s: form 0 staged (5 kernels), 1 fused warp kernel,
-// 2 plain CTA-per-frame kernel; forms 0 and 1 finish with the deferred-frame
-// kernel.  Timing events are recorded when `timed`.
+// Whether a call that asks for the staged form takes a CTA per frame instead (the same
+// decisions): a small batch of a decision-only run, for which two launches and one frame's
+// latency replace eight launches and two memsets.
+bool takes_small(int form, int64_t n, bool debug, bool timed, const void* stats) {
+  return form == FORM_STAGED && n <= SMALL_FRAMES && !debug && !timed && !stats;
+}
+
+// Enqueue one batch on stream s: form 0 staged (5 kernels; small batches a CTA per frame
+// unless `small` is false), 1 fused warp kernel, 2 plain CTA-per-frame kernel; forms 0 and
+// 1 finish with the deferred-frame kernel.  Timing events are recorded when `timed`.
 int enqueue(m3e_ctx* x, Scratch& sc, KParams p, int form, bool debug, cudaStream_t s, bool timed,
-            cudaEvent_t after_s1 = nullptr) {
+            cudaEvent_t after_s1 = nullptr, bool small = true) {
+  if (small && !p.gate && takes_small(form, p.n_frames, debug, timed, p.stats)) {
+    CUDA_TRY(launch_small(x->dc, p, x->sms, s));
+    x->last_launches = 2;
+    return M3E_OK;
+  }
+  // frames per queue grab: at least two grabs for every resident warp, so that a batch of
+  // a few frames per warp spreads over all of them
+  const int64_t warps = (int64_t)x->sms * WARPS_PER_CTA * (form == FORM_FUSED ? x->fused_bpsm : x->s1_bpsm);
+  p.grab = (int)std::max<int64_t>(1, std::min<int64_t>(p.grab, p.n_frames / (2 * warps)));
   if (form == FORM_PLAIN) {
     if (timed) CUDA_TRY(cudaEventRecord(x->pe[0], s));
     CUDA_TRY(launch_plain(x->dc, p, debug, s));
@@ -589,7 +605,8 @@ static int select_common(m3e_ctx* x, const int32_t* hits, const int64_t* off, in
   x->prof_valid = false;
   if (n == 0) return M3E_OK;
   DeviceGuard guard(x->device);
-  rc = ensure_scratch(x->main, n, form == FORM_STAGED);
+  const bool timed = x->prof && dump == nullptr;
+  if (!takes_small(form, n, dump != nullptr, timed, stats)) rc = ensure_scratch(x->main, n, form == FORM_STAGED);
   if (rc) return rc;
   KParams p = base_params(x, x->main);
   p.hits = hits;
@@ -606,7 +623,6 @@ static int select_common(m3e_ctx* x, const int32_t* hits, const int64_t* off, in
       return fail(M3E_EINVAL, "incomplete m3e_dump");
     p.dump = *dump;
   }
-  const bool timed = x->prof && dump == nullptr;
   rc = enqueue(x, x->main, p, form, dump != nullptr, s, timed);
   x->prof_valid = timed && rc == M3E_OK;
   x->prof_kind = form;
@@ -837,6 +853,17 @@ extern "C" int m3e_select_frames_noalloc(m3e_ctx* x, const int32_t* d_hits, cons
   x->prof_valid = false;
   if (n_frames == 0) return M3E_OK;
   DeviceGuard guard(x->device);
+  if (n_frames <= SMALL_FRAMES) {  // no scratch at all
+    KParams ps = base_params(x, x->main);
+    ps.hits = d_hits;
+    ps.off = d_frame_off;
+    ps.n_frames = n_frames;
+    ps.keep = d_keep;
+    ps.reason = d_reason;
+    CUDA_TRY(launch_small(x->dc, ps, x->sms, s));
+    x->last_launches = 2;
+    return M3E_OK;
+  }
   int* scratch = nullptr;
   rc = noalloc_scratch(x->device, &scratch);
   if (rc) return rc;
@@ -973,10 +1000,10 @@ extern "C" int m3e_autotune(m3e_ctx* x, const int32_t* d_hits, const int64_t* d_
     p.keep = d_keep;
     p.reason = d_reason;
     float t[5];
-    int r = enqueue(x, x->main, p, FORM_STAGED, false, st, false);  // warm-up
+    int r = enqueue(x, x->main, p, FORM_STAGED, false, st, false, nullptr, false);  // warm-up
     for (int k = 0; k < 5 && r == M3E_OK; ++k) {
       CUDA_TRY(cudaEventRecord(e0, st));
-      r = enqueue(x, x->main, p, FORM_STAGED, false, st, false);
+      r = enqueue(x, x->main, p, FORM_STAGED, false, st, false, nullptr, false);
       CUDA_TRY(cudaEventRecord(e1, st));
       CUDA_TRY(cudaEventSynchronize(e1));
       CUDA_TRY(cudaEventElapsedTime(&t[k], e0, e1));

@@ -100,6 +100,13 @@ __device__ __forceinline__ void cp_async4(void* smem_dst, const void* gsrc) {
   const unsigned d = (unsigned)__cvta_generic_to_shared(smem_dst);
   asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(d), "l"(gsrc) : "memory");
 }
+// Programmatic dependent launch.  pdl_wait: wait until the preceding kernel of the stream
+// has finished and its writes are visible (nothing to wait for in an ordinary launch);
+// every block of a kernel launched with launch_pdl calls it before it reads or writes
+// memory.  pdl_trigger: the following kernel's blocks may be placed once every block of
+// this one has got here or ended.
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void prefetch_l1(const void* p) {
   asm volatile("prefetch.global.L1 [%0];" ::"l"(p));
 }
@@ -1497,9 +1504,9 @@ __device__ int frame_front(const G& g, S& sm, const DevCfg& C, const KParams& P,
 
 // Stages D-F of one frame after frame_front returned PENDING: track
 // reconstruction, energy test and vertex.  Returns a final reason or DEFERRED.
-template <class G, class S, int CT, int CK, int CC, bool DEFER, bool DEBUG>
+template <class G, class S, int CT, int CK, int CC, bool DEFER, bool DEBUG, bool NOST = false>
 __device__ int frame_back(const G& g, S& sm, const DevCfg& C, const KParams& P, int f) {
-  const bool stats = P.stats != nullptr;
+  const bool stats = !NOST && P.stats != nullptr;
   const int ntrip = sm.ntrip;
   const SmHits<S> view{sm};
   // ---- D: track reconstruction (Algorithm 3), one thread per triplet
@@ -1651,6 +1658,23 @@ template <class G, class S>
 __device__ __forceinline__ void clear_stats(const G& g, S& sm) {
   for (int k = g.rank(); k < ST_REASON0 + 8; k += G::N) sm.acc[k] = 0;
   g.sync();
+}
+
+// Launch with programmatic stream serialisation: the launch and the prologue overlap the
+// end of the kernel before it on the stream.
+template <class... K, class... A>
+cudaError_t launch_pdl(void (*k)(K...), int grid, int threads, size_t smem, cudaStream_t s, const A&... a) {
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3((unsigned)grid);
+  cfg.blockDim = dim3((unsigned)threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, k, a...);
 }
 
 }  // namespace

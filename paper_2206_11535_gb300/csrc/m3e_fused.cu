@@ -66,6 +66,57 @@ __global__ void __launch_bounds__(NT) k_select_cta(const __grid_constant__ DevCf
   flush_stats(g, sm, P.stats);
 }
 
+// Small batches: a CTA per frame with a stage of 512 hits, so that a whole small batch is
+// resident at once and the call takes one frame's latency.  A frame beyond the stage is
+// marked in its reason for k_select_marked.
+using SmSmall = FrameSm<SMALL_HITS, SMALL_TRIP, C_TRK, C_COMBO>;
+constexpr uint8_t MARK = 0xff;
+
+// NT: threads of a CTA, CTAS: of them per SM.  Measured (us, batches of nominal / throughput /
+// 32-track frames): 64 frames 14 / 19 / 23 with 256 threads, 14 / 23 / 32 with 128; 2048
+// frames 35 / 54 / 72 against 24 / 47 / 70.  The wide CTAs serve batches that they hold
+// resident at once.
+template <int NT, int CTAS>
+__global__ void __launch_bounds__(NT, CTAS)
+    k_select_small(const __grid_constant__ DevCfg C, const __grid_constant__ KParams P) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  SmSmall& sm = *reinterpret_cast<SmSmall*>(smem_raw);
+  const CtaGroup<NT> g;
+  pdl_trigger();
+  const int f = blockIdx.x;
+  int r = frame_front<CtaGroup<NT>, SmSmall, SMALL_HITS, SMALL_TRIP, true, false, false, true>(g, sm, C, P, f);
+  if (r == PENDING)
+    r = frame_back<CtaGroup<NT>, SmSmall, SMALL_TRIP, C_TRK, C_COMBO, true, false, true>(g, sm, C, P, f);
+  if (r != DEFERRED) finish_frame<CtaGroup<NT>, SmSmall, true>(g, sm, P, f, r);
+  else if (g.leader()) P.reason[f] = MARK;
+}
+
+// The frames that k_select_small marked, with the stage of the configuration limits; one
+// look at the marks per thread (the grid has a thread for every frame of a small batch).
+__global__ void __launch_bounds__(CTA_THREADS)
+    k_select_marked(const __grid_constant__ DevCfg C, const __grid_constant__ KParams P) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  SmCta& sm = *reinterpret_cast<SmCta*>(smem_raw);
+  __shared__ int list[CTA_THREADS];
+  __shared__ int count;
+  const CtaGroup<CTA_THREADS> g;
+  if (g.leader()) count = 0;
+  pdl_wait();
+  __syncthreads();
+  const int64_t mine = blockIdx.x + (int64_t)gridDim.x * threadIdx.x;
+  if (mine < P.n_frames && P.reason[mine] == MARK) list[atomicAdd(&count, 1)] = (int)mine;
+  __syncthreads();
+  const int n = count;
+  for (int i = 0; i < n; ++i) {
+    const int f = list[i];
+    int r = frame_front<CtaGroup<CTA_THREADS>, SmCta, C_HITS, C_TRIP, false, false, false, true>(g, sm, C, P, f);
+    if (r == PENDING)
+      r = frame_back<CtaGroup<CTA_THREADS>, SmCta, C_TRIP, C_TRK, C_COMBO, false, false, true>(g, sm, C, P, f);
+    finish_frame<CtaGroup<CTA_THREADS>, SmCta, true>(g, sm, P, f, r);
+    g.sync();
+  }
+}
+
 template <class K>
 cudaError_t set_smem(K k, size_t bytes) {
   return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
@@ -111,6 +162,19 @@ cudaError_t launch_deferred(const DevCfg& c, const KParams& p, int grid, bool de
     k_select_cta<CTA_THREADS, false, true><<<grid, CTA_THREADS, sm, s>>>(c, p);
   }
   return cudaGetLastError();
+}
+
+// A batch of at most SMALL_FRAMES frames (no scratch, no counters to clear).
+cudaError_t launch_small(const DevCfg& c, KParams p, int sms, cudaStream_t s) {
+  p.defer_hits = SMALL_HITS;
+  const bool wide = p.n_frames <= 4 * sms;
+  cudaError_t e = wide ? set_smem(k_select_small<256, 4>, sizeof(SmSmall)) : set_smem(k_select_small<128, 8>, sizeof(SmSmall));
+  if (e == cudaSuccess) e = set_smem(k_select_marked, sizeof(SmCta));
+  if (e != cudaSuccess) return e;
+  if (wide) k_select_small<256, 4><<<(int)p.n_frames, 256, sizeof(SmSmall), s>>>(c, p);
+  else k_select_small<128, 8><<<(int)p.n_frames, 128, sizeof(SmSmall), s>>>(c, p);
+  const int grid = (int)(p.n_frames < 2 * sms ? p.n_frames : 2 * sms);
+  return launch_pdl(k_select_marked, grid, CTA_THREADS, sizeof(SmCta), s, c, p);
 }
 
 cudaError_t launch_plain(const DevCfg& c, const KParams& p, bool debug, cudaStream_t s) {

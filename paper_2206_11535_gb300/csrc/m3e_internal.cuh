@@ -24,6 +24,13 @@ constexpr int C_HITS = 4096, C_TRIP = 1024, C_TRK = 128, C_COMBO = 1024;
 constexpr int WARPS_PER_CTA = 4;  // persistent warp kernel: warps (frames in flight) per CTA
 constexpr int CTA_THREADS = 256;  // large-frame kernel
 constexpr int PLAIN_THREADS = 128;  // plain per-frame kernel
+// Small batches: a CTA per frame, its stage sized for eight CTAs per SM.  Up to how many
+// frames: against the staged form 2048 nominal frames take 24 and 62 us, throughput frames 47
+// and 92, 32-track frames 70 and 142, uneven ones 167 and 261; 8192 of them 78 and 77, 149 and
+// 128, 237 and 219, 405 and 323.  Only frames of 64 tracks, most of which overflow, cross
+// earlier (1000 frames 263 and 256, 2048 430 and 345).
+constexpr int SMALL_HITS = 512, SMALL_TRIP = 512;
+constexpr int64_t SMALL_FRAMES = 2048;
 
 // Geometry and cuts, precomputed on the host in FP64 and rounded once.
 struct DevCfg {
@@ -111,6 +118,7 @@ enum { ERR_BADHIT = 1, ERR_NEGSIZE = 2, ERR_GATE = 4 };
 // Host-side launchers (m3e_fused.cu, m3e_staged.cu).
 cudaError_t launch_fused(const DevCfg& c, const KParams& p, int grid, bool debug, cudaStream_t s);
 cudaError_t launch_deferred(const DevCfg& c, const KParams& p, int grid, bool debug, cudaStream_t s);
+cudaError_t launch_small(const DevCfg& c, KParams p, int sms, cudaStream_t s);
 cudaError_t launch_plain(const DevCfg& c, const KParams& p, bool debug, cudaStream_t s);
 cudaError_t launch_staged(const DevCfg& c, const KParams& p, const SParams& s, const int grids[6], bool debug,
                           cudaStream_t st, cudaEvent_t* ev, cudaEvent_t after_s1 = nullptr, int mid_threads = 256);
