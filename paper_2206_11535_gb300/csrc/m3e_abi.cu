@@ -74,7 +74,6 @@ struct Scratch {
   int* defer1b = nullptr;                   // list 1b (staged form)
   int64_t defer_cap = 0;
   float* hf = nullptr;                      // hx, hy, hz, hphi
-  uint32_t* haddr = nullptr;
   uint16_t* hidx = nullptr;
   int64_t hits_cap = 0;
   uint16_t* l3 = nullptr;
@@ -309,10 +308,9 @@ int ensure_scratch(Scratch& sc, int64_t nf, bool staged) {
   if (!staged) return M3E_OK;
   int64_t hc = sc.hits_cap;
   if (nh > hc) {
-    int64_t c0 = hc, c1 = hc, c2 = hc;
+    int64_t c0 = hc, c1 = hc;
     rc = grow(sc.hf, c0, nh, 4 * sizeof(float), "sorted hits");
-    if (!rc) rc = grow(sc.haddr, c1, nh, sizeof(uint32_t), "sorted addresses");
-    if (!rc) rc = grow(sc.hidx, c2, nh, sizeof(uint16_t), "sorted input indices");
+    if (!rc) rc = grow(sc.hidx, c1, nh, sizeof(uint16_t), "sorted input indices");
     if (rc) return rc;
     sc.hits_cap = nh;
   }
@@ -344,7 +342,6 @@ void free_scratch(Scratch& sc) {
   cudaFree(sc.defer2);
   cudaFree(sc.defer1b);
   cudaFree(sc.hf);
-  cudaFree(sc.haddr);
   cudaFree(sc.hidx);
   cudaFree(sc.l3);
   cudaFree(sc.fint);
@@ -360,7 +357,6 @@ SParams staged_params(const Scratch& sc) {
   SParams s{};
   const int64_t H = sc.hits_cap, F = sc.frames_cap;
   s.hp = reinterpret_cast<float4*>(sc.hf);
-  s.haddr = sc.haddr;
   s.hidx = sc.hidx;
   s.l3 = sc.l3;
   s.fstate = sc.fint;

@@ -52,26 +52,28 @@ struct TrkSoA {
   int tid[CK];                      // index of the triplet it came from
 };
 
-// PHI / IDX: whether the stage keeps each hit's phi (the layer-3 search of the
-// fused track stage reads it) and its input index (candidate record only); a
-// stage without them holds more frames in flight per SM.  Triplets of a stage of
-// at most 256 hits are kept as 8-bit indices.
-template <int CH, int CT, int CK, int CC, bool PHI = true, bool IDX = true, bool ADDR = true,
-          int CH32 = (CH <= W_HITS ? CH : 1)>
+// IDX: whether the stage keeps each hit's input index (candidate record only); STATS:
+// whether it has room for statistics.  A stage without them holds more frames in flight
+// per SM.  Triplets of a stage of at most 256 hits are kept as 8-bit indices.
+template <int CH, int CT, int CK, int CC, bool IDX = true, bool STATS = true, int CH32 = (CH <= W_HITS ? CH : 1)>
 struct FrameSm {
-  static constexpr bool kPhi = PHI, kIdx = IDX, kAddr = ADDR;
+  static constexpr bool kIdx = IDX, kStats = STATS;
   static constexpr bool kPackB = CH < 256;  // bucket cursors as bytes, four to a word
   using TripT = typename std::conditional<(CH <= 256), uchar4, ushort4>::type;
-  float x[CH], y[CH], z[CH], phi[PHI ? CH : 1];
-  uint32_t addr[ADDR ? CH : 1];
+  alignas(16) float x[CH];
+  alignas(16) float y[CH];
+  float z[CH], phi[CH];         // phi: layer-3 hits only (the 4th-hit search)
   uint16_t inidx[IDX ? CH : 1];
   uint16_t bstart[NBK + 1];
   uint32_t bcur[kPackB ? NBK / 4 : NBK];  // bucket counts, then cursors
   // warp stage, selection cuts (warp_cuts): the layer-2 hits in z-bin order (bin
-  // starts zbs), the (layer-1 hit, Phi01 partner) pairs of a chunk of 32 layer-1 hits
-  // (their layer-0 hits) and the candidate triplets of one round of pairs
-  float4 zq[CH32 == 1 ? 1 : W_L2];  // layer-2 hits in z-bin order: x, y, z, sorted index (as int bits)
-  uint8_t p01[CH32 == 1 ? 1 : W_P01];
+  // starts zbs; z and sorted index in zzi), the (layer-1 hit, Phi01 partner) pairs of a
+  // chunk of 32 layer-1 hits (layer-0 hit, lane of the layer-1 hit) and the candidate
+  // triplets of one round of pairs
+  alignas(16) float zx[CH32 == 1 ? 4 : W_L2];
+  alignas(16) float zy[CH32 == 1 ? 4 : W_L2];
+  float2 zzi[CH32 == 1 ? 1 : W_L2];
+  uint16_t p01[CH32 == 1 ? 1 : W_P01];
   uint8_t zbs[CH32 == 1 ? 1 : NZB + 1];
   alignas(16) uint16_t cand[CH32 == 1 ? 1 : W_CAND];  // also the z-bin counters (32-bit words)
   // CTA stage, selection cuts: the layer-2 hits in z-bin order (sorted-hit indices),
@@ -85,14 +87,38 @@ struct FrameSm {
     uint32_t combo[CC];         // e+ e+ e- combinations (track indices), after the fits
   } u;
   int ntrip, npos, nneg, ncombo, nstore, flag, bad;
-  unsigned long long acc[ST_REASON0 + 8];  // statistics of this group's frames
-  unsigned long long facc[ST_REASON0];     // statistics of the current frame
+  unsigned long long acc[STATS ? ST_REASON0 + 8 : 1];  // statistics of this group's frames
+  unsigned long long facc[STATS ? ST_REASON0 : 1];     // statistics of the current frame
 };
 
 using SmWarp = FrameSm<W_HITS, W_TRIP, W_TRK, W_COMBO>;
 using SmCta = FrameSm<C_HITS, C_TRIP, C_TRK, C_COMBO>;
 
 // ------------------------------------------------------------------ small helpers
+
+// Two FP32 operations in one instruction, each rounded as the scalar one.
+__device__ __forceinline__ unsigned long long pack2(float lo, float hi) {
+  unsigned long long r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+  return r;
+}
+__device__ __forceinline__ unsigned long long mul2(unsigned long long a, unsigned long long b) {
+  unsigned long long r;
+  asm("mul.rn.ftz.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ unsigned long long fma2(unsigned long long a, unsigned long long b, unsigned long long c) {
+  unsigned long long r;
+  asm("fma.rn.ftz.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+__device__ __forceinline__ unsigned long long add2(unsigned long long a, unsigned long long b) {
+  unsigned long long r;
+  asm("add.rn.ftz.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+// The bits below bit k of a word, all 32 for k of 32 and more (k >= 0).
+__device__ __forceinline__ uint32_t bits_below(int k) { return __funnelshift_lc(0xffffffffu, 0u, (unsigned)k); }
 
 // Asynchronous 4-byte copy from global to shared memory (no register holds the
 // value), and the wait for all of this thread's copies.
@@ -363,7 +389,6 @@ struct SmHits {
   static constexpr bool kPark = false;
   const S& s;
   __device__ __forceinline__ float4 pos(int i) const { return make_float4(s.x[i], s.y[i], s.z[i], s.phi[i]); }
-  __device__ __forceinline__ uint32_t addr(int i) const { return s.addr[i]; }
   __device__ __forceinline__ int l3(int b) const { return s.bstart[3 * NB + b]; }  // layer-3 bin starts
 };
 
@@ -412,11 +437,9 @@ __device__ __forceinline__ TFitF unpark_fit(const FitPark& pk) {
 struct GHits {                       // one 16-byte load per hit
   static constexpr bool kPark = true;
   const float4* __restrict__ ps;
-  const uint32_t* __restrict__ as;
   const uint16_t* __restrict__ l3s;  // NB + 1 layer-3 bin starts, frame-relative
   FitPark* park;
   __device__ __forceinline__ float4 pos(int i) const { return __ldg(ps + i); }
-  __device__ __forceinline__ uint32_t addr(int i) const { return __ldg(as + i); }
   __device__ __forceinline__ int l3(int b) const { return __ldg(l3s + b); }
 };
 
@@ -513,7 +536,6 @@ __device__ __forceinline__ TrackOut build_track(const V& v, const DevCfg& C, int
   b3 = b3 < 0 ? 0 : (b3 >= NB ? NB - 1 : b3);
   int best = -1;
   float mb = FLT_MAX;
-  uint32_t ab = 0;
   // (r3 dphi)^2 + dz^2, rounded in one fixed order wherever it is inlined; dphi is
   // the difference of the azimuths (both in [0, 2 pi)) less the nearest multiple of
   // 2 pi, which one fused multiply-add subtracts exactly as a subtraction of 2 pi
@@ -524,15 +546,20 @@ __device__ __forceinline__ TrackOut build_track(const V& v, const DevCfg& C, int
     const float dz = __fsub_rn(q.z, z3);
     return __fmaf_rn(rd, rd, __fmul_rn(dz, dz));
   };
-  // the full rule: an equal metric goes to the smaller address
+  // the full rule: an equal metric goes to the smaller address.  The address orders the
+  // layer's hits by column, then row, and the coordinates grow with these (a column's phi,
+  // a row's z), so the comparison needs no address
   auto visit = [&](int j) {
     const float4 q = v.pos(j);
-    const uint32_t aj = v.addr(j);
     const float mm = metric(q);
-    if (best < 0 || mm < mb || (mm == mb && aj < ab)) {
+    bool take = best < 0 || mm < mb;
+    if (mm == mb && !take) {
+      const float4 o = v.pos(best);
+      take = q.w < o.w || (q.w == o.w && q.z < o.z);
+    }
+    if (take) {
       best = j;
       mb = mm;
-      ab = aj;
     }
   };
   const int l3a = v.l3(0), l3e = v.l3(NB);
@@ -993,6 +1020,28 @@ __device__ __forceinline__ void bucket_scan(const G& g, S& sm) {
   g.sync();
 }
 
+// Which of n <= 32 hits (xs, ys: 16-byte aligned, readable to the next multiple of four)
+// pass the Phi cut with the hit whose coordinates xx, yy hold twice: bit q for hit q.  The
+// test is phi_pass, two hits per instruction; the sign of (product - c), which is exact, is
+// shifted into the mask, the last hit first.
+__device__ __forceinline__ uint32_t phi_mask(const float* xs, const float* ys, int n, unsigned long long xx,
+                                             unsigned long long yy, float c) {
+  const unsigned long long mc = pack2(-c, -c);
+  uint32_t m = 0u;
+#pragma unroll 2
+  for (int q = ((n + 3) & ~3) - 4; q >= 0; q -= 4) {
+    const ulonglong2 X = *reinterpret_cast<const ulonglong2*>(xs + q);
+    const ulonglong2 Y = *reinterpret_cast<const ulonglong2*>(ys + q);
+    const unsigned long long t1 = add2(fma2(X.y, xx, mul2(Y.y, yy)), mc);
+    const unsigned long long t0 = add2(fma2(X.x, xx, mul2(Y.x, yy)), mc);
+    m = __funnelshift_l((uint32_t)(t1 >> 32), m, 1);
+    m = __funnelshift_l((uint32_t)t1, m, 1);
+    m = __funnelshift_l((uint32_t)(t0 >> 32), m, 1);
+    m = __funnelshift_l((uint32_t)t0, m, 1);
+  }
+  return ~m & bits_below(n);
+}
+
 // Selection cuts of a warp-stage frame (Algorithm 2), on the hits sorted by (layer,
 // phi bin).  The layer-2 hits are also put in z-bin order (x, y, z and index packed
 // in one record), so that for a (layer-1 hit, Phi01 partner) pair the Delta lambda
@@ -1059,7 +1108,9 @@ __device__ __forceinline__ void warp_cuts(S& sm, const DevCfg& C, bool stats, un
       if (bq >= 0) {
         const int i2 = l1b + lane + 32 * h;
         const int pos = (int)((atomicAdd(&zc[bq >> 2], 1u << (8 * (bq & 3))) >> (8 * (bq & 3))) & 255u);
-        sm.zq[pos] = make_float4(sm.x[i2], sm.y[i2], sm.z[i2], __int_as_float(i2));
+        sm.zx[pos] = sm.x[i2];
+        sm.zy[pos] = sm.y[i2];
+        sm.zzi[pos] = make_float2(sm.z[i2], __int_as_float(i2));
       }
     }
     __syncwarp();
@@ -1085,20 +1136,11 @@ __device__ __forceinline__ void warp_cuts(S& sm, const DevCfg& C, bool stats, un
     }
     // 1. Phi01 and Phi12 partners as bit masks (lanes without a layer-1 hit test
     // (0, 0), which passes neither cut)
-    uint32_t a0 = 0u, a1 = 0u, b0 = 0u, b1 = 0u;
-    const int n0a = min(n0, 32), n2a = min(n2, 32);
-    for (int q = 0; q < n0a; ++q)
-      if (phi_pass(sm.x[q], sm.y[q], x1, y1, C.c01)) a0 |= 1u << q;
-    for (int q = 32; q < n0; ++q)
-      if (phi_pass(sm.x[q], sm.y[q], x1, y1, C.c01)) a1 |= 1u << (q - 32);
-    for (int q = 0; q < n2a; ++q) {
-      const float4 h = sm.zq[q];
-      if (phi_pass(x1, y1, h.x, h.y, C.c12)) b0 |= 1u << q;
-    }
-    for (int q = 32; q < n2; ++q) {
-      const float4 h = sm.zq[q];
-      if (phi_pass(x1, y1, h.x, h.y, C.c12)) b1 |= 1u << (q - 32);
-    }
+    const unsigned long long xx = pack2(x1, x1), yy = pack2(y1, y1);
+    const uint32_t a0 = phi_mask(sm.x, sm.y, min(n0, 32), xx, yy, C.c01);
+    const uint32_t a1 = n0 > 32 ? phi_mask(sm.x + 32, sm.y + 32, n0 - 32, xx, yy, C.c01) : 0u;
+    const uint32_t b0 = phi_mask(sm.zx, sm.zy, min(n2, 32), xx, yy, C.c12);
+    const uint32_t b1 = n2 > 32 ? phi_mask(sm.zx + 32, sm.zy + 32, n2 - 32, xx, yy, C.c12) : 0u;
     const int c01 = __popc(a0) + __popc(a1), c12all = __popc(b0) + __popc(b1);
     ntt += (unsigned)(c01 * c12all);
     // 2. the pairs whose layer-1 hit has Phi12 partners, listed by their layer-0 hit
@@ -1117,38 +1159,30 @@ __device__ __forceinline__ void warp_cuts(S& sm, const DevCfg& C, bool stats, un
     }
     if (pc) {
       int wpos = pre;
-      for (uint32_t m = a0; m; m &= m - 1u) sm.p01[wpos++] = (uint8_t)(__ffs(m) - 1);
-      for (uint32_t m = a1; m; m &= m - 1u) sm.p01[wpos++] = (uint8_t)(__ffs(m) + 31);
+      for (uint32_t m = a0; m; m &= m - 1u) sm.p01[wpos++] = (uint16_t)((__ffs(m) - 1) | (lane << 8));
+      for (uint32_t m = a1; m; m &= m - 1u) sm.p01[wpos++] = (uint16_t)((__ffs(m) + 31) | (lane << 8));
     }
     __syncwarp();
     // 3. the pairs, 32 at a time
     for (int k0 = 0; k0 < T; k0 += 32) {
       const int k = k0 + lane;
-      int ow = 0;  // the last lane whose pairs start at or before k
-#pragma unroll
-      for (int st = 16; st; st >>= 1) {
-        const int pv = __shfl_sync(FULL, pre, ow + st);
-        if (pv <= k) ow += st;
-      }
+      const int pair = k < T ? sm.p01[k] : 0;
+      const int i0 = pair & 255, ow = pair >> 8;  // layer-0 hit, lane of the layer-1 hit
       const float px1 = __shfl_sync(FULL, x1, ow), py1 = __shfl_sync(FULL, y1, ow), pz1 = __shfl_sync(FULL, z1, ow);
-      const uint32_t pml = __shfl_sync(FULL, b0, ow), pmh = __shfl_sync(FULL, b1, ow);
-      int i0 = 0;
-      float x0 = 0.f, y0 = 0.f, tl01 = 0.f;
-      unsigned long long cm = 0ull;
+      uint32_t cl = __shfl_sync(FULL, b0, ow), ch = 0u;
+      if (n2 > 32) ch = __shfl_sync(FULL, b1, ow);
+      const float x0 = sm.x[i0], y0 = sm.y[i0], tl01 = tan_l01(sm.z[i0], pz1, C);
+      int lo = 0, hi = 0;
       if (k < T) {
-        i0 = sm.p01[k];
-        x0 = sm.x[i0];
-        y0 = sm.y[i0];
-        tl01 = tan_l01(sm.z[i0], pz1, C);
         const float zlo = pz1 + (tl01 - C.dl_max) * C.dr12 - 1e-3f;
         const float zhi = pz1 + (tl01 + C.dl_max) * C.dr12 + 1e-3f;
-        const int lo = sm.zbs[zbin2(zlo, C)], hi = sm.zbs[zbin2(zhi, C) + 1];
-        const unsigned long long below_hi = hi >= 64 ? ~0ull : (1ull << hi) - 1ull;
-        const unsigned long long below_lo = lo >= 64 ? ~0ull : (1ull << lo) - 1ull;
-        cm = (below_hi & ~below_lo) & (((unsigned long long)pmh << 32) | pml);
+        lo = sm.zbs[zbin2(zlo, C)];
+        hi = sm.zbs[zbin2(zhi, C) + 1];
       }
+      cl &= bits_below(hi) & ~bits_below(lo);
+      if (n2 > 32) ch &= bits_below(max(hi - 32, 0)) & ~bits_below(max(lo - 32, 0));
       const int tri01 = i0 | ((l1a + j0 + ow) << 8);  // the pair's layer-0 and layer-1 sorted indices
-      const int cnt = __popcll(cm);
+      const int cnt = __popc(cl) + __popc(ch);
       int ce = cnt;
 #pragma unroll
       for (int o = 1; o < 32; o <<= 1) {
@@ -1158,11 +1192,15 @@ __device__ __forceinline__ void warp_cuts(S& sm, const DevCfg& C, bool stats, un
       const int cpre = ce - cnt, ctot = __shfl_sync(FULL, ce, 31);
       for (int c0 = 0; c0 < ctot; c0 += W_CAND) {
         // each lane lists its candidates numbered c0 .. c0 + W_CAND - 1: pair lane, z-order position
-        unsigned long long m = cm;
-        for (int idx = cpre; m; ++idx) {
-          const int q = __ffsll((long long)m) - 1;
-          m &= m - 1ull;
-          if (idx >= c0 && idx < c0 + W_CAND) sm.cand[idx - c0] = (uint16_t)((lane << 6) | q);
+        int idx = cpre - c0;
+        if (ctot <= W_CAND) {  // all of them fit: the usual case
+          for (uint32_t m = cl; m; m &= m - 1u) sm.cand[idx++] = (uint16_t)((lane << 6) | (__ffs(m) - 1));
+          for (uint32_t m = ch; m; m &= m - 1u) sm.cand[idx++] = (uint16_t)((lane << 6) | (__ffs(m) + 31));
+        } else {
+          for (uint32_t m = cl; m; m &= m - 1u, ++idx)
+            if (idx >= 0 && idx < W_CAND) sm.cand[idx] = (uint16_t)((lane << 6) | (__ffs(m) - 1));
+          for (uint32_t m = ch; m; m &= m - 1u, ++idx)
+            if (idx >= 0 && idx < W_CAND) sm.cand[idx] = (uint16_t)((lane << 6) | (__ffs(m) + 31));
         }
         __syncwarp();
         // 4. the exact tests, 32 candidates at a time
@@ -1175,11 +1213,12 @@ __device__ __forceinline__ void warp_cuts(S& sm, const DevCfg& C, bool stats, un
           const float cx1 = __shfl_sync(FULL, px1, pl), cy1 = __shfl_sync(FULL, py1, pl);
           const float cz1 = __shfl_sync(FULL, pz1, pl), ctl = __shfl_sync(FULL, tl01, pl);
           const int ct = __shfl_sync(FULL, tri01, pl);
-          const float4 h = sm.zq[ent & 63];
-          const bool pass = e < ne && dl_pass(cz1, h.z, ctl, C) && rtc_pass(cx0, cy0, cx1, cy1, h.x, h.y, C);
+          const float2 h = sm.zzi[ent & 63];
+          const bool pass = e < ne && dl_pass(cz1, h.x, ctl, C) &&
+                            rtc_pass(cx0, cy0, cx1, cy1, sm.zx[ent & 63], sm.zy[ent & 63], C);
           const unsigned bm = __ballot_sync(FULL, pass);
           const int kk = nt + __popc(bm & ((1u << lane) - 1u));
-          if (pass && kk < CT) sm.u.trip[kk] = make_trip<typename S::TripT>(ct & 255, ct >> 8, __float_as_int(h.w));
+          if (pass && kk < CT) sm.u.trip[kk] = make_trip<typename S::TripT>(ct & 255, ct >> 8, __float_as_int(h.y));
           nt += __popc(bm);
         }
         __syncwarp();
@@ -1240,9 +1279,9 @@ __device__ int frame_front(const G& g, S& sm, const DevCfg& C, const KParams& P,
   for (int k = g.rank(); k < (S::kPackB ? NBK / 4 : NBK); k += G::N) sm.bcur[k] = 0;
   // warp stage: the per-layer decode table (DevCfg::ltab) for parts A and B, in the
   // space of the layer-2 z order, which part C fills later
-  uint4* const ltab = reinterpret_cast<uint4*>(sm.zq);
+  uint4* const ltab = reinterpret_cast<uint4*>(sm.zx);
   if constexpr (G::N == 32 && DEFER && TAB) {
-    static_assert(sizeof(sm.zq) >= 4 * sizeof(uint4), "room for the decode table");
+    static_assert(sizeof(sm.zx) >= 4 * sizeof(uint4), "room for the decode table");
     if (g.rank() < 4) ltab[g.rank()] = C.ltab[g.rank()];
   }
   if (g.leader()) {
@@ -1268,13 +1307,17 @@ __device__ int frame_front(const G& g, S& sm, const DevCfg& C, const KParams& P,
       const int i = lane + 32 * k;
       av[k] = i < n ? (uint32_t)(LIVE ? __ldcv(hp + i) : __ldg(hp + i)) : 0u;
     }
+    // the bucket and the table indices (15 bits each) of a hit stay in registers
     bool bad = false;
+    int key[K];
 #pragma unroll
     for (int k = 0; k < K; ++k) {
       if (lane + 32 * k < n) {
         const Dec d = TAB ? decode_s(ltab, av[k]) : decode(C, av[k]);
+        key[k] = d.L * NB + d.b;
+        av[k] = (uint32_t)d.ci | (uint32_t)d.ri << 15;
         if (!d.ok) bad = true;
-        else bucket_add(sm, d.L * NB + d.b);
+        else bucket_add(sm, key[k]);
       }
     }
     if (__any_sync(FULL, bad)) {
@@ -1293,14 +1336,12 @@ __device__ int frame_front(const G& g, S& sm, const DevCfg& C, const KParams& P,
     for (int k = 0; k < K; ++k) {
       const int i = lane + 32 * k;
       if (i < n) {
-        const Dec d = TAB ? decode_s(ltab, av[k]) : decode(C, av[k]);
-        const int pos = bucket_add(sm, d.L * NB + d.b);
-        const float* cl = reinterpret_cast<const float*>(P.col_lut + d.ci);
+        const int pos = bucket_add(sm, key[k]);
+        const float* cl = reinterpret_cast<const float*>(P.col_lut + (av[k] & 0x7fffu));
         cp_async4(&sm.x[pos], cl);
         cp_async4(&sm.y[pos], cl + 1);
-        if constexpr (S::kPhi) cp_async4(&sm.phi[pos], cl + 2);
-        cp_async4(&sm.z[pos], P.row_lut + d.ri);
-        if constexpr (S::kAddr) sm.addr[pos] = av[k];
+        if (key[k] >= 3 * NB) cp_async4(&sm.phi[pos], cl + 2);
+        cp_async4(&sm.z[pos], P.row_lut + (av[k] >> 15));
         if constexpr (S::kIdx) sm.inidx[pos] = (uint16_t)i;
       }
     }
@@ -1332,9 +1373,8 @@ __device__ int frame_front(const G& g, S& sm, const DevCfg& C, const KParams& P,
       const float4 c4 = __ldg(P.col_lut + d.ci);
       sm.x[pos] = c4.x;
       sm.y[pos] = c4.y;
-      if constexpr (S::kPhi) sm.phi[pos] = c4.z;
+      sm.phi[pos] = c4.z;
       sm.z[pos] = __ldg(P.row_lut + d.ri);
-      if constexpr (S::kAddr) sm.addr[pos] = a;
       if constexpr (S::kIdx) sm.inidx[pos] = (uint16_t)i;
     }
   }

@@ -15,7 +15,7 @@ namespace {
 // the device work queue; a frame that outgrows the warp's shared-memory stage is
 // appended to the deferred list for the CTA kernel.
 template <bool DEBUG>
-__global__ void __launch_bounds__(WARPS_PER_CTA * 32)
+__global__ void __launch_bounds__(WARPS_PER_CTA * 32, 5)  // as many CTAs per SM as its shared memory allows
     k_select_warp(const __grid_constant__ DevCfg C, const __grid_constant__ KParams P) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   SmWarp& sm = reinterpret_cast<SmWarp*>(smem_raw)[threadIdx.x >> 5];

@@ -92,7 +92,6 @@ struct KParams {
 // Global scratch of the staged form (see m3e_staged.cu), sized per batch.
 struct SParams {
   float4* hp;                  // sorted hits of the pending frames (from the hit allocator): x, y, z, phi
-  uint32_t* haddr;
   uint16_t* hidx;              // input index of each sorted hit (candidate record only)
   int* list1;                  // frames deferred by the warp tier of stage 1
   int* list1b;                 // frames deferred by the middle tier of stage 1

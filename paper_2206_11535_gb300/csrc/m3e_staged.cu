@@ -18,10 +18,11 @@ namespace {
 
 constexpr int NL3 = NB + 1;                        // layer-3 bin starts per frame
 constexpr int S1_TRIP = 160;                       // stage-1 warp-tier triplet capacity
-// the address of each hit at hand for the emit (its phi is computed there); input
-// indices only for the candidate record
-using SmFront = FrameSm<W_HITS, S1_TRIP, 1, 1, false, false, true>;
-using SmFrontD = FrameSm<W_HITS, S1_TRIP, 1, 1, false, true, true>;
+// input indices only for the candidate record; the instance without statistics code has
+// no room for them
+using SmFrontN = FrameSm<W_HITS, S1_TRIP, 1, 1, false, false>;
+using SmFront = FrameSm<W_HITS, S1_TRIP, 1, 1, false>;
+using SmFrontD = FrameSm<W_HITS, S1_TRIP, 1, 1>;
 constexpr int M_HITS = 1024;                       // stage-1 middle tier (CTA per frame)
 using SmFrontMid = FrameSm<M_HITS, C_TRIP, 1, 1>;
 using SmFrontCta = FrameSm<C_HITS, C_TRIP, 1, 1>;
@@ -50,31 +51,16 @@ __device__ __forceinline__ int warp_count_add(int* ctr, bool pred) {  // ordered
 // onwards, so no allocator is needed); its triplets go to a range taken from the
 // triplet allocator, whose atomic is issued first and waited for only after the
 // hits are written.  A frame that does not fit is deferred (returns false).
-template <class G, class Sm, bool DEBUG, bool LIVE = false>
+template <class G, class Sm, bool DEBUG>
 __device__ __forceinline__ bool emit_frame(const G& g, Sm& sm, const DevCfg& C, const KParams& P, const SParams& S,
                                            int f, int n, int ntrip, long long* bcast) {
   long long tb = 0;
   if (g.leader()) tb = (long long)atomicAdd(&S.counters[0], (unsigned long long)ntrip);
   const long long hb = P.off[f] - P.off_base;
   const bool hits_fit = hb + n <= S.hits_cap;
-  // phi and the address of a sorted hit serve only the layer-3 search of stage 2
-  const int l3s = sm.bstart[3 * NB];
-  const int32_t* hin = P.hits + hb;
+  const int l3s = sm.bstart[3 * NB];  // phi of a sorted hit serves only the layer-3 search of stage 2
   for (int i = g.rank(); hits_fit && i < n; i += G::N) {
-    float phi = 0.f;
-    if (i >= l3s) {
-      uint32_t a;
-      if constexpr (Sm::kAddr) a = sm.addr[i];
-      else a = (uint32_t)(LIVE ? __ldcv(hin + sm.inidx[i]) : __ldg(hin + sm.inidx[i]));
-      if constexpr (Sm::kPhi) {
-        phi = sm.phi[i];
-      } else {
-        const Dec d = decode(C, a);
-        phi = column_phi(C, d.L, d.g);
-      }
-      S.haddr[hb + i] = a;
-    }
-    S.hp[hb + i] = make_float4(sm.x[i], sm.y[i], sm.z[i], phi);
+    S.hp[hb + i] = make_float4(sm.x[i], sm.y[i], sm.z[i], i >= l3s ? sm.phi[i] : 0.f);
     if constexpr (DEBUG) {
       static_assert(Sm::kIdx, "the candidate record needs the input indices");
       S.hidx[hb + i] = sm.inidx[i];
@@ -108,14 +94,14 @@ __device__ __forceinline__ bool emit_frame(const G& g, Sm& sm, const DevCfg& C, 
 }
 
 // After frame_front: decide, emit, or defer one frame (stage-1 tiers).
-template <class G, class Sm, bool DEBUG, bool LIVE = false, bool NOST = false>
+template <class G, class Sm, bool DEBUG, bool NOST = false>
 __device__ __forceinline__ void stage1_finish(const G& g, Sm& sm, const DevCfg& C, const KParams& P, const SParams& S,
                                               int f, int r, long long* bcast) {
   const int ntrip = sm.ntrip;
   if (r == PENDING && ntrip == 0) r = M3E_DROP;  // no triplet: no track, no vertex
   if (r == PENDING) {
     const int n = (int)(P.off[f + 1] - P.off[f]);
-    if (emit_frame<G, Sm, DEBUG, LIVE>(g, sm, C, P, S, f, n, ntrip, bcast)) {
+    if (emit_frame<G, Sm, DEBUG>(g, sm, C, P, S, f, n, ntrip, bcast)) {
       if (!NOST && g.leader() && P.stats)
         for (int k = 0; k < ST_REASON0; ++k) sm.acc[k] += sm.facc[k];
     } else {
@@ -174,15 +160,19 @@ __device__ bool gate_wait(const KParams& P, int k) {
 // GATED (host entry point): the hits arrive while the kernel runs; a frame is
 // taken only after its chunk's arrival flag, and the hits are read past L1.
 // NOST: the instance for runs without statistics (no statistics code at all).
+// Bound by instruction issue and shared-memory latency (1,934 warp instructions per
+// throughput frame at 66% issue active; l1tex 68% busy with the table gathers): 1e6
+// throughput frames 2.36 -> 2.15 ms with the packed partner masks, one decode per hit and no
+// address list, at 64 registers and 8 CTAs per SM (2.20 ms at 56 registers and 9 CTAs).
 template <bool DEBUG, bool GATED = false, bool NOST = false>
 __global__ void __launch_bounds__(WARPS_PER_CTA * 32)
     k_stage1(const __grid_constant__ DevCfg C, const __grid_constant__ KParams P, const __grid_constant__ SParams S) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  using Sm = typename std::conditional<DEBUG, SmFrontD, SmFront>::type;
+  using Sm = typename std::conditional<DEBUG, SmFrontD, typename std::conditional<NOST, SmFrontN, SmFront>::type>::type;
   Sm& sm = reinterpret_cast<Sm*>(smem_raw)[threadIdx.x >> 5];
   __shared__ long long bcast[WARPS_PER_CTA][2];
   const WarpGroup g;
-  clear_stats(g, sm);
+  if (!NOST) clear_stats(g, sm);
   const int nf = (int)P.n_frames;
   int arrived = -1;  // chunks up to this one are known to have arrived
   bool stop = false;
@@ -204,7 +194,7 @@ __global__ void __launch_bounds__(WARPS_PER_CTA * 32)
         }
       }
       const int r = frame_front<WarpGroup, Sm, W_HITS, S1_TRIP, true, DEBUG, GATED, NOST, true>(g, sm, C, P, f, f + 1 < f1);
-      stage1_finish<WarpGroup, Sm, DEBUG, GATED, NOST>(g, sm, C, P, S, f, r, bcast[threadIdx.x >> 5]);
+      stage1_finish<WarpGroup, Sm, DEBUG, NOST>(g, sm, C, P, S, f, r, bcast[threadIdx.x >> 5]);
     }
   }
   if (!NOST) flush_stats(g, sm, P.stats);
@@ -227,7 +217,7 @@ __global__ void __launch_bounds__(NT)
     int r;
     if (CH < C_HITS && P.off[f + 1] - P.off[f] > CH) r = DEFERRED;  // for the next tier
     else r = frame_front<CtaGroup<NT>, Sm, CH, C_TRIP, false, DEBUG, false, NOST>(g, sm, C, P, f);
-    stage1_finish<CtaGroup<NT>, Sm, DEBUG, false, NOST>(g, sm, C, P, S, f, r, bcast);
+    stage1_finish<CtaGroup<NT>, Sm, DEBUG, NOST>(g, sm, C, P, S, f, r, bcast);
   }
   if (!NOST) flush_stats(g, sm, P.stats);
 }
@@ -251,7 +241,7 @@ __global__ void __launch_bounds__(128, 8)  // 8 CTAs per SM (64 registers: the f
     if (f < 0) continue;
     const int64_t base = (int64_t)(unsigned)r.y;
     const int i0 = r.z & 0xffff, i1 = (int)((unsigned)r.z >> 16), i2 = r.w;
-    const GHits v{S.hp + base, S.haddr + base, S.l3 + (int64_t)f * NL3, &park};
+    const GHits v{S.hp + base, S.l3 + (int64_t)f * NL3, &park};
     const TrackOut o = build_track(v, C, i0, i1, i2);
     float2 te = make_float2(0.f, 0.f);
     if (o.status == 5) {
@@ -591,7 +581,9 @@ cudaError_t set_smem(K k, size_t bytes) {
 
 }  // namespace
 
-size_t stage1_smem_bytes(bool debug = false) { return (debug ? sizeof(SmFrontD) : sizeof(SmFront)) * WARPS_PER_CTA; }
+size_t stage1_smem_bytes(bool debug, bool nost) {
+  return (debug ? sizeof(SmFrontD) : nost ? sizeof(SmFrontN) : sizeof(SmFront)) * WARPS_PER_CTA;
+}
 size_t stage1c_smem_bytes() { return sizeof(SmFrontCta); }
 size_t stage1m_smem_bytes() { return sizeof(SmFrontMid); }
 
@@ -599,9 +591,9 @@ int stage_blocks_per_sm(int stage) {
   int nb = 0;
   cudaError_t e = cudaSuccess;
   if (stage == 1) {
-    set_smem(k_stage1<false, false, true>, stage1_smem_bytes());
+    set_smem(k_stage1<false, false, true>, stage1_smem_bytes(false, true));
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_stage1<false, false, true>, WARPS_PER_CTA * 32,
-                                                      stage1_smem_bytes());
+                                                      stage1_smem_bytes(false, true));
   } else if (stage == 2) {
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_stage2<false>, 128, 0);
   } else if (stage == 3) {
@@ -656,9 +648,9 @@ cudaError_t launch_tier(const DevCfg& c, const KParams& p, const SParams& s, int
 
 cudaError_t launch_staged(const DevCfg& c, const KParams& p, const SParams& s, const int grids[6], bool debug,
                           cudaStream_t st, cudaEvent_t* ev, cudaEvent_t after_s1, int mid_threads) {
-  const size_t sm1 = stage1_smem_bytes(debug), smc = stage1c_smem_bytes(), smm = stage1m_smem_bytes();
   const bool gated = p.gate != nullptr && !debug;
   const bool nost = p.stats == nullptr;
+  const size_t sm1 = stage1_smem_bytes(debug, nost), smc = stage1c_smem_bytes(), smm = stage1m_smem_bytes();
   cudaError_t e = debug ? set_smem(k_stage1<true>, sm1)
                   : gated ? (nost ? set_smem(k_stage1<false, true, true>, sm1) : set_smem(k_stage1<false, true>, sm1))
                           : (nost ? set_smem(k_stage1<false, false, true>, sm1) : set_smem(k_stage1<false>, sm1));
