@@ -77,7 +77,7 @@ struct Scratch {
   uint16_t* hidx = nullptr;
   int64_t hits_cap = 0;
   uint16_t* l3 = nullptr;
-  int* fint = nullptr;                      // fstate, ftbase, fntrip, ffound, fncombo
+  int* fint = nullptr;                      // fstate, ftbase, fntrip, ffound
   long long* fcbase = nullptr;              // per frame: first combination
   int64_t frames_cap = 0;
   int4* trip = nullptr;
@@ -317,7 +317,7 @@ int ensure_scratch(Scratch& sc, int64_t nf, bool staged) {
   if (nf > sc.frames_cap) {
     int64_t c0 = sc.frames_cap, c1 = sc.frames_cap, c2 = sc.frames_cap;
     rc = grow(sc.l3, c0, nf, (NB + 1) * sizeof(uint16_t), "layer-3 bins");
-    if (!rc) rc = grow(sc.fint, c1, nf, 5 * sizeof(int), "frame state");
+    if (!rc) rc = grow(sc.fint, c1, nf, 4 * sizeof(int), "frame state");
     if (!rc) rc = grow(sc.fcbase, c2, nf, sizeof(long long), "frame combination bases");
     if (rc) return rc;
     sc.frames_cap = nf;
@@ -363,7 +363,6 @@ SParams staged_params(const Scratch& sc) {
   s.ftbase = sc.fint + F;
   s.fntrip = sc.fint + 2 * F;
   s.ffound = sc.fint + 3 * F;
-  s.fncombo = sc.fint + 4 * F;
   s.fcbase = sc.fcbase;
   s.list1 = sc.defer;
   s.list2 = sc.defer2;

@@ -924,6 +924,97 @@ __device__ __forceinline__ VtxOut vertex(const TrackR& A, const TrackR& B, const
   return o;
 }
 
+// ------------------------------------------------------------------ energy test
+
+// The pr-th pair (a, b), a < b, of the order (0,1), (0,2), (1,2), (0,3), ...: the root is
+// exact to one unit for every pair of C_TRK tracks, and each side is corrected once.
+__device__ __forceinline__ void pair_of(int pr, int& a, int& b) {
+  b = (int)((1.f + sqrtf(1.f + 8.f * (float)pr)) * 0.5f);
+  if (b * (b - 1) / 2 > pr) --b;
+  if ((b + 1) * b / 2 <= pr) ++b;
+  a = pr - b * (b - 1) / 2;
+}
+
+// Energy test of every (e+ pair, e-) combination of a frame by one warp (Algorithm 4,
+// part 1), a pair per lane and two e- at a time (two sums per instruction).  pEP: E and
+// p cos(theta) of each e+ track; nEP: the e- tracks two by two, E of c and c + 1, then
+// p cos(theta) of c and c + 1, an odd last track paired with a NaN energy, which passes no
+// window.  Counts the combinations passing (ncombo) and, with stats, those whose P_z leaves
+// the momentum cut open (nopen); put(k, a, b, c) gets the k-th combination to fit, in
+// (pair, e-) order: all that pass, or with prune the open ones.  Once more than `enough`
+// passed the frame overflows whatever follows, and the rest is not looked at.
+template <class Put>
+__device__ __forceinline__ void energy_test(const DevCfg& C, const float2* pEP, const float4* nEP, int npos, int nneg,
+                                            bool prune, bool stats, int enough, int& ncombo, int& nwrite, int& nopen, const Put& put) {
+  const int lane = threadIdx.x & 31;
+  const unsigned below = (1u << lane) - 1u;
+  const int npair = npos * (npos - 1) / 2;
+  const unsigned long long mmu = pack2(-C.m_mu, -C.m_mu);
+  for (int p0 = 0; p0 < npair && ncombo <= enough; p0 += 32) {
+    const int pr = p0 + lane;
+    int a = 0, b = 0;
+    float eab = __int_as_float(0x7fc00000), pzab = 0.f;  // NaN: a lane without a pair passes no window
+    if (pr < npair) {
+      pair_of(pr, a, b);
+      const float2 ta = pEP[a], tb = pEP[b];
+      eab = ta.x + tb.x;
+      pzab = __fadd_rn(ta.y, tb.y);
+    }
+    const unsigned long long e2 = pack2(eab, eab), z2 = pack2(pzab, pzab);
+    int cnt = 0, co = 0;
+    for (int c = 0; c < nneg; c += 2) {
+      const ulonglong2 v = *reinterpret_cast<const ulonglong2*>(nEP + (c >> 1));
+      const unsigned long long d = add2(add2(e2, v.x), mmu), z = add2(z2, v.y);
+      const bool ok0 = fabsf(__uint_as_float((unsigned)d)) <= C.e_win;
+      const bool ok1 = fabsf(__uint_as_float((unsigned)(d >> 32))) <= C.e_win;
+      cnt += ok0;
+      cnt += ok1;
+      const bool open0 = ok0 && !pz_fails_ptot(__uint_as_float((unsigned)z), C.ptot_max);
+      const bool open1 = ok1 && !pz_fails_ptot(__uint_as_float((unsigned)(z >> 32)), C.ptot_max);
+      const bool wr0 = prune ? open0 : ok0, wr1 = prune ? open1 : ok1;
+      if (__any_sync(FULL, wr0 || wr1)) {
+        co += open0;
+        co += open1;
+        const unsigned m0 = __ballot_sync(FULL, wr0), m1 = __ballot_sync(FULL, wr1);
+        if (wr0) put(nwrite + __popc(m0 & below), a, b, c);
+        if (wr1) put(nwrite + __popc(m0) + __popc(m1 & below), a, b, c + 1);
+        nwrite += __popc(m0) + __popc(m1);
+      }
+    }
+    ncombo += __reduce_add_sync(FULL, cnt);
+    if (stats) nopen += __reduce_add_sync(FULL, co);
+  }
+}
+
+// Kept tracks of 32 triplets into the lists of energy_test (te: (eps E, P_z) of this lane's
+// triplet, E > 0, or (0, 0)); put(k, positive) gets the place of this lane's track.
+template <class Put>
+__device__ __forceinline__ void list_tracks(const float2& te, float2* pEP, float4* nEP, int cap, int& npos, int& nneg,
+                                            const Put& put) {
+  const unsigned below = (1u << (threadIdx.x & 31)) - 1u;
+  const bool pos = te.x > 0.f, neg = te.x < 0.f;
+  const unsigned mp = __ballot_sync(FULL, pos), mn = __ballot_sync(FULL, neg);
+  const int kp = npos + __popc(mp & below), kn = nneg + __popc(mn & below);
+  npos += __popc(mp);
+  nneg += __popc(mn);
+  if (pos && kp < cap) {
+    pEP[kp] = te;
+    put(kp, true);
+  }
+  if (neg && kn < cap) {
+    float* q = reinterpret_cast<float*>(nEP + (kn >> 1)) + (kn & 1);
+    q[0] = -te.x;
+    q[2] = te.y;
+    put(kn, false);
+  }
+}
+// The NaN beside an odd last e- track; then the lists are complete.
+__device__ __forceinline__ void close_lists(float4* nEP, int cap, int nneg) {
+  if ((threadIdx.x & 31) == 0 && (nneg & 1) && nneg < cap)
+    reinterpret_cast<float*>(nEP + (nneg >> 1))[1] = __int_as_float(0x7fc00000);
+  __syncwarp();
+}
+
 // ------------------------------------------------------------------ one frame
 
 
@@ -1594,10 +1685,10 @@ __device__ int frame_back(const G& g, S& sm, const DevCfg& C, const KParams& P, 
   {
     const int npair = npos * (npos - 1) / 2;
     for (int pr = g.rank(); pr < npair; pr += G::N) {
-      int b = (int)((1.f + sqrtf(1.f + 8.f * (float)pr)) * 0.5f);
-      while (b * (b - 1) / 2 > pr) --b;
-      while ((b + 1) * b / 2 <= pr) ++b;
-      const int a = pr - b * (b - 1) / 2;
+      // past the cap the decision is known (the candidate record wants the full count)
+      if (!DEBUG && *(volatile int*)&sm.ncombo > C.max_combo) break;
+      int a, b;
+      pair_of(pr, a, b);
       const float eab = sm.t.E[a] + sm.t.E[b];
       const float pzab = __fadd_rn(pz_track(sm.t.p[a], sm.t.ct[a]), pz_track(sm.t.p[b], sm.t.ct[b]));
       for (int c = 0; c < nneg; ++c) {

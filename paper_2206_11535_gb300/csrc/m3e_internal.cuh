@@ -99,8 +99,7 @@ struct SParams {
   int* lcount;                 // [0] list1 count, [1] list2 count, [2] list1b count
   uint16_t* l3;                // [F][NB + 1] layer-3 phi-bin starts, frame-relative
   int *fstate, *ftbase, *fntrip, *ffound;  // per frame: state, triplet range, vertex found
-  long long* fcbase;           // per frame: first combination
-  int* fncombo;
+  long long* fcbase;           // per frame: first combination (candidate record only)
   int4* trip;                  // {frame, first sorted hit, i0 | i1 << 16, i2} (frame-relative indices), frame -1 = unused
   float2* tek;                 // per triplet: (eps E, P_z) of a kept track, (0, 0) otherwise
   float4* trec;                // per triplet: 16-float track record when kept

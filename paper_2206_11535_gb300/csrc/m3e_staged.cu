@@ -11,6 +11,8 @@
 // instructions and lanes; a frame's candidates stay contiguous, so its hits and
 // tracks are read from L2 by neighbouring threads.  Frames that exceed a stage's
 // capacity are deferred to the CTA-per-frame kernel with identical decisions.
+#include <algorithm>
+
 #include "m3e_device.cuh"
 
 namespace m3e {
@@ -27,24 +29,17 @@ constexpr int M_HITS = 1024;                       // stage-1 middle tier (CTA p
 using SmFrontMid = FrameSm<M_HITS, C_TRIP, 1, 1>;
 using SmFrontCta = FrameSm<C_HITS, C_TRIP, 1, 1>;
 constexpr int S3_WARPS = 4;
-constexpr int S3_BUF = 128;  // combinations a frame of stage 3 collects before writing
+constexpr int S3_BUF = 96;   // combinations a warp of stage 3 collects before writing
+constexpr int S3_CHUNK = 4;  // frames a warp of stage 3 takes at a time, at most
 
+template <bool STATS>
 struct S3Sm {                                      // stage 3, per warp
-  int pidx[C_TRK], nidx[C_TRK];                    // triplet index of each e+ / e- track
-  float pE[C_TRK], nE[C_TRK];
-  float pPz[C_TRK], nPz[C_TRK];                    // p cos(theta) of each track
-  uint32_t wbuf[S3_BUF];                           // combinations to write: a | b << 8 | c << 16
-  int npos, nneg;
-  unsigned long long acc[ST_REASON0 + 8];
+  float4 nEP[C_TRK / 2];                           // tracks as energy_test reads them
+  float2 pEP[C_TRK];
+  uint16_t pidx[C_TRK], nidx[C_TRK];               // triplet of each, counted in its frame
+  int4 buf[S3_BUF];                                // combinations to write
+  unsigned long long acc[STATS ? ST_REASON0 + 8 : 1];
 };
-
-__device__ __forceinline__ int warp_count_add(int* ctr, bool pred) {  // ordered warp compaction
-  const unsigned m = __ballot_sync(FULL, pred);
-  int base = 0;
-  if ((threadIdx.x & 31) == 0 && m) base = atomicAdd(ctr, __popc(m));
-  base = __shfl_sync(FULL, base, 0);
-  return base + __popc(m & ((1u << (threadIdx.x & 31)) - 1u));
-}
 
 // ---- stage 1: write-out of a frame whose cuts selected triplets
 // The sorted hits of frame f take the places of its input hits (off[f] - off_base
@@ -274,169 +269,157 @@ __global__ void __launch_bounds__(128, 8)  // 8 CTAs per SM (64 registers: the f
 }
 
 // ---- stage 3: warp per frame, track cap and energy test (NOST: the instance for
-// runs without statistics)
+// runs without statistics).
+// A warp takes P.grab frames at a time: their states are read together, a lane each, the
+// tracks of the next frame are loaded while one is tested, and the combinations of all of
+// them are written behind one allocation, a fourth of the atomics on the one counter.
+// Bound by issue (770 warp instructions per throughput frame, 73% issue active, 10 CTAs per
+// SM at 48 registers; 12 spill and take 15% longer): 1e6 throughput frames 854 -> 719 us,
+// 200,000 uneven frames 541 -> 283 us, most of that from frames that stop at the combination
+// cap.  Taking 16 frames at a time cost 745 and 535 us (heavy frames queue in one warp).
 template <bool DEBUG, bool NOST = false>
-__global__ void __launch_bounds__(S3_WARPS * 32)
+__global__ void __launch_bounds__(S3_WARPS * 32, 10)
     k_stage3(const __grid_constant__ DevCfg C, const __grid_constant__ KParams P, const __grid_constant__ SParams S) {
-  __shared__ S3Sm smem[S3_WARPS];
-  S3Sm& sm = smem[threadIdx.x >> 5];
+  __shared__ S3Sm<!NOST> smem[S3_WARPS];
+  S3Sm<!NOST>& sm = smem[threadIdx.x >> 5];
   const int lane = threadIdx.x & 31;
-  for (int k = lane; k < ST_REASON0 + 8; k += 32) sm.acc[k] = 0;
+  if (!NOST)
+    for (int k = lane; k < ST_REASON0 + 8; k += 32) sm.acc[k] = 0;
   __syncwarp();
   const int nf = (int)P.n_frames;
   const bool stats = !NOST && P.stats != nullptr;
+  // all energy-test survivors count towards the cap; a decision-only run writes only those
+  // whose P_z leaves the momentum cut open (pz_fails_ptot)
+  const bool prune = !DEBUG && !stats;
   for (;;) {
     int f0 = 0;
     if (lane == 0) f0 = (int)atomicAdd(&S.counters[2], (unsigned long long)P.grab);
     f0 = __shfl_sync(FULL, f0, 0);
     if (f0 >= nf) break;
-    const int f1 = min(f0 + P.grab, nf);
-    for (int f = f0; f < f1; ++f) {
-      if (S.fstate[f] != PENDING) continue;
-      const int tb = S.ftbase[f], nt = S.fntrip[f];
-      if (lane == 0) {
-        sm.npos = 0;
-        sm.nneg = 0;
+    // this lane's frame: state, triplet range, decision taken here, combinations collected
+    const int f = f0 + lane;
+    const bool mine = lane < P.grab && f < nf;
+    int tbase = 0, ntrip = 0, r = PENDING, at = -1, stat_combo = 0, stat_open = 0;
+    bool pending = false;
+    if (mine) {
+      pending = S.fstate[f] == PENDING;
+      tbase = S.ftbase[f];
+      ntrip = S.fntrip[f];
+    }
+    unsigned todo = __ballot_sync(FULL, pending);
+    int fill = 0;  // combinations in the buffer
+    auto load = [&](int j, int t) {  // (eps E, P_z) of triplet t + lane of lane j's frame, (0, 0) beyond them
+      const int tb = __shfl_sync(FULL, tbase, j), nt = __shfl_sync(FULL, ntrip, j);
+      return t + lane < nt ? __ldg(S.tek + tb + t + lane) : make_float2(0.f, 0.f);
+    };
+    // n combinations get a range of the scratch: its start, or -1 when it is full
+    auto allocate = [&](int n) -> long long {
+      long long cb = 0;
+      if (lane == 0) cb = (long long)atomicAdd(&S.counters[1], (unsigned long long)n);
+      cb = __shfl_sync(FULL, cb, 0);
+      if (cb + n <= S.combo_cap) return cb;
+      for (int64_t t = cb + lane; t < S.combo_cap; t += 32) S.combo[t] = make_int4(-1, 0, 0, 0);
+      return -1;
+    };
+    // frames whose combinations went to the range at cb (at: this lane's place in it), or found no room
+    auto placed = [&](long long cb) {
+      if (at < 0) return;
+      if (cb < 0) {
+        r = DEFERRED;
+      } else {
+        if (DEBUG) S.fcbase[f] = cb + at;
+        if (stats) {
+          atomicAdd(&sm.acc[ST_COMBO], (unsigned long long)stat_combo);
+          atomicAdd(&sm.acc[ST_PZOPEN], (unsigned long long)stat_open);
+        }
       }
+      at = -1;
+    };
+    auto flush = [&]() {
+      if (fill == 0) return;
       __syncwarp();
+      const long long cb = allocate(fill);
+      for (int t = lane; cb >= 0 && t < fill; t += 32) S.combo[cb + t] = sm.buf[t];
+      placed(cb);
+      fill = 0;
+      __syncwarp();
+    };
+    float2 n0 = make_float2(0.f, 0.f), n1 = n0;
+    if (todo) {
+      n0 = load(__ffs(todo) - 1, 0);
+      n1 = load(__ffs(todo) - 1, 32);
+    }
+    while (todo) {
+      const int j = __ffs(todo) - 1;
+      todo &= todo - 1u;
+      const int tb = __shfl_sync(FULL, tbase, j), nt = __shfl_sync(FULL, ntrip, j), fj = f0 + j;
+      const float2 te0 = n0, te1 = n1;
+      if (todo) {
+        n0 = load(__ffs(todo) - 1, 0);
+        n1 = load(__ffs(todo) - 1, 32);
+      }
       // kept tracks of the frame's triplets, split by charge
-      for (int t0 = 0; t0 < nt; t0 += 32) {
-        const int t = t0 + lane;
-        // (eps E, P_z) of a kept track (E > 0), (0, 0) for a triplet that made none
-        const float2 te = t < nt ? __ldg(S.tek + tb + t) : make_float2(0.f, 0.f);
-        const float E = fabsf(te.x), pz = te.y;
-        const bool pos = te.x > 0.f, neg = te.x < 0.f;
-        const int kp = warp_count_add(&sm.npos, pos);
-        const int kn = warp_count_add(&sm.nneg, neg);
-        if (pos && kp < C_TRK) {
-          sm.pidx[kp] = tb + t;
-          sm.pE[kp] = E;
-          sm.pPz[kp] = pz;
-        }
-        if (neg && kn < C_TRK) {
-          sm.nidx[kn] = tb + t;
-          sm.nE[kn] = E;
-          sm.nPz[kn] = pz;
-        }
-        __syncwarp();
-      }
-      __syncwarp();
-      const int npos = sm.npos, nneg = sm.nneg;
-      int r = PENDING;
-      if (npos + nneg > C.max_trk) r = M3E_TRACK_OVERFLOW;
-      const int npair = npos * (npos - 1) / 2;
-      // all energy-test survivors count towards the cap; a decision-only run
-      // writes only those whose P_z leaves the momentum cut open (pz_fails_ptot)
-      const bool prune = !DEBUG && !stats;
-      int ncombo = 0, nwrite = 0, nopen = 0;
-      if (r == PENDING) {
+      int npos = 0, nneg = 0;
+      auto list = [&](const float2& te, int t0) {
+        list_tracks(te, sm.pEP, sm.nEP, C_TRK, npos, nneg,
+                    [&](int k, bool pos) { (pos ? sm.pidx : sm.nidx)[k] = (uint16_t)(t0 + lane); });
+      };
+      list(te0, 0);
+      if (nt > 32) list(te1, 32);
+      for (int t0 = 64; t0 < nt; t0 += 32) list(load(j, t0), t0);
+      close_lists(sm.nEP, C_TRK, nneg);
+      int rj = PENDING, ncombo = 0, nopen = 0, nw = fill;
+      if (npos + nneg > C.max_trk) rj = M3E_TRACK_OVERFLOW;
+      if (rj == PENDING) {
         if (stats && lane == 0) {
           sm.acc[ST_TRK] += npos + nneg;
-          sm.acc[ST_ETEST] += (unsigned long long)npair * nneg;
+          sm.acc[ST_ETEST] += (unsigned long long)(npos * (npos - 1) / 2) * nneg;
         }
-        // one pass over the (e+ pair, e-) combinations: count those passing the energy
-        // test and collect those to write, in (pair, e-) order, in the warp's buffer
-        for (int p0 = 0; p0 < npair; p0 += 32) {
-          const int pr = p0 + lane;
-          const bool act = pr < npair;
-          int a = 0, b = 0;
-          float eab = 0.f, pzab = 0.f;
-          if (act) {
-            b = (int)((1.f + sqrtf(1.f + 8.f * (float)pr)) * 0.5f);
-            while (b * (b - 1) / 2 > pr) --b;
-            while ((b + 1) * b / 2 <= pr) ++b;
-            a = pr - b * (b - 1) / 2;
-            eab = sm.pE[a] + sm.pE[b];
-            pzab = __fadd_rn(sm.pPz[a], sm.pPz[b]);
+        auto record = [&](int a, int b, int c) {
+          return make_int4(fj, tb + sm.pidx[a], tb + sm.pidx[b], tb + sm.nidx[c]);
+        };
+        energy_test(C, sm.pEP, sm.nEP, npos, nneg, prune, stats, DEBUG ? 1 << 30 : C.max_combo, ncombo, nw, nopen,
+                    [&](int k, int a, int b, int c) {
+                      if (k < S3_BUF) sm.buf[k] = record(a, b, c);
+                    });
+        if (DEBUG && lane == 0) P.dump.n_combo[fj] = ncombo;
+        if (ncombo > C.max_combo) rj = M3E_COMBO_OVERFLOW;
+        else if (nw == fill) rj = M3E_DROP;  // no combination, or none that can pass
+        else {
+          const int own = nw - fill;
+          const bool fits = nw <= S3_BUF;
+          if (!fits) flush();
+          if (lane == j) {
+            at = fill;
+            stat_combo = ncombo;
+            stat_open = nopen;
           }
-          int cnt = 0, co = 0;
-          for (int c = 0; c < nneg; ++c) {
-            const bool e_ok = act && fabsf((eab + sm.nE[c]) - C.m_mu) <= C.e_win;
-            cnt += e_ok;
-            // few combinations pass the energy window: the P_z test and the write
-            // run only for an e- where one of the warp's pairs passes
-            if (__any_sync(FULL, e_ok)) {
-              const bool open = e_ok && !pz_fails_ptot(__fadd_rn(pzab, sm.nPz[c]), C.ptot_max);
-              co += open;
-              const bool wr = prune ? open : e_ok;
-              const unsigned m = __ballot_sync(FULL, wr);
-              const int k = nwrite + __popc(m & ((1u << lane) - 1u));
-              if (wr && k < S3_BUF) sm.wbuf[k] = (uint32_t)a | ((uint32_t)b << 8) | ((uint32_t)c << 16);
-              nwrite += __popc(m);
-            }
-          }
-          ncombo += __reduce_add_sync(FULL, cnt);
-          if (stats) nopen += __reduce_add_sync(FULL, co);
-        }
-        __syncwarp();
-        if (DEBUG && lane == 0) P.dump.n_combo[f] = ncombo;
-        if (ncombo > C.max_combo) r = M3E_COMBO_OVERFLOW;
-        else if (nwrite == 0) r = M3E_DROP;  // no combination, or none that can pass
-      }
-      if (r == PENDING) {
-        long long cb = 0;
-        if (lane == 0) cb = (long long)atomicAdd(&S.counters[1], (unsigned long long)nwrite);
-        cb = __shfl_sync(FULL, cb, 0);
-        if (cb + nwrite > S.combo_cap) {
-          for (int64_t t = cb + lane; t < S.combo_cap; t += 32) S.combo[t] = make_int4(-1, 0, 0, 0);
-          r = DEFERRED;
-        } else {
-          if (nwrite <= S3_BUF) {
-            for (int t = lane; t < nwrite; t += 32) {
-              const uint32_t v = sm.wbuf[t];
-              S.combo[cb + t] = make_int4(f, sm.pidx[v & 255], sm.pidx[(v >> 8) & 255], sm.nidx[v >> 16]);
-            }
+          if (fits) {
+            fill = nw;
           } else {
-            // more than the buffer holds: a second pass writes them, in the same order
-            long long w = cb;
-            for (int p0 = 0; p0 < npair; p0 += 32) {
-              const int pr = p0 + lane;
-              int a = 0, b = 0;
-              float eab = 0.f, pzab = 0.f;
-              const bool act = pr < npair;
-              if (act) {
-                b = (int)((1.f + sqrtf(1.f + 8.f * (float)pr)) * 0.5f);
-                while (b * (b - 1) / 2 > pr) --b;
-                while ((b + 1) * b / 2 <= pr) ++b;
-                a = pr - b * (b - 1) / 2;
-                eab = sm.pE[a] + sm.pE[b];
-                pzab = __fadd_rn(sm.pPz[a], sm.pPz[b]);
-              }
-              for (int c = 0; c < nneg; ++c) {
-                const bool pass = act && fabsf((eab + sm.nE[c]) - C.m_mu) <= C.e_win &&
-                                  !(prune && pz_fails_ptot(__fadd_rn(pzab, sm.nPz[c]), C.ptot_max));
-                const unsigned m = __ballot_sync(FULL, pass);
-                if (pass) S.combo[w + __popc(m & ((1u << lane) - 1u))] = make_int4(f, sm.pidx[a], sm.pidx[b], sm.nidx[c]);
-                w += __popc(m);
-              }
-            }
-          }
-          if (lane == 0) {
-            S.fcbase[f] = cb;
-            S.fncombo[f] = nwrite;
-            if (stats) {
-              sm.acc[ST_COMBO] += ncombo;
-              sm.acc[ST_PZOPEN] += nopen;
-            }
+            // not beside the earlier ones: a second pass writes this frame's, in the same order
+            const long long cb = allocate(own);
+            int again = 0, c1 = 0, c2 = 0;
+            if (cb >= 0)
+              energy_test(C, sm.pEP, sm.nEP, npos, nneg, prune, false, 1 << 30, c1, again, c2,
+                          [&](int k, int a, int b, int c) { S.combo[cb + k] = record(a, b, c); });
+            placed(cb);
           }
         }
       }
-      if (r == DEFERRED) {
-        if (lane == 0) {
-          S.fstate[f] = DEFERRED;
-          const int k = atomicAdd(P.defer_count, 1);
-          P.defer_list[k] = f;
-          if (stats) sm.acc[ST_DEFER] += 1;
-        }
-      } else if (r != PENDING) {
-        if (lane == 0) {
-          S.fstate[f] = r;
-          P.keep[f] = (uint8_t)(r != M3E_DROP);
-          P.reason[f] = (uint8_t)r;
-          if (stats) sm.acc[ST_REASON0 + r] += 1;
-        }
-      }
+      if (lane == j) r = rj == PENDING ? r : rj;
       __syncwarp();
+    }
+    flush();
+    if (pending && r == DEFERRED) {
+      S.fstate[f] = DEFERRED;
+      P.defer_list[atomicAdd(P.defer_count, 1)] = f;
+      if (stats) atomicAdd(&sm.acc[ST_DEFER], 1ull);
+    } else if (pending && r != PENDING) {
+      S.fstate[f] = r;
+      P.keep[f] = (uint8_t)(r != M3E_DROP);
+      P.reason[f] = (uint8_t)r;
+      if (stats) atomicAdd(&sm.acc[ST_REASON0 + r], 1ull);
     }
   }
   __syncwarp();
@@ -517,7 +500,7 @@ __global__ void __launch_bounds__(S4_WARPS * 32, 8)  // 8 CTAs per SM (64 regist
         load_circle(S.trec, r.y, ca[0], ca[1], ca[2]);
         load_circle(S.trec, r.z, cb[0], cb[1], cb[2]);
         load_circle(S.trec, r.w, ce[0], ce[1], ce[2]);
-        if (S.fstate[f] == PENDING && (DEBUG || !*((volatile int*)S.ffound + f))) {
+        if (DEBUG || !*((volatile int*)S.ffound + f)) {
           const int st = vertex_prefilter(ca, cb, ce, C.isect_lim);
           cand = st == 2;
           if (DEBUG && !cand) {  // record the combination with its early status (the same geometry)
@@ -668,6 +651,8 @@ cudaError_t launch_staged(const DevCfg& c, const KParams& p, const SParams& s, c
   pc.defer_count = s.lcount + 1;
   p3.defer_list = s.list2;
   p3.defer_count = s.lcount + 1;
+  // frames a warp of stage 3 takes at a time: two takes for every resident warp
+  p3.grab = (int)std::max<int64_t>(1, std::min<int64_t>(S3_CHUNK, p.n_frames / (2 * (int64_t)grids[2] * S3_WARPS)));
   if (ev) cudaEventRecord(ev[0], st);
   if (debug) k_stage1<true><<<grids[0], WARPS_PER_CTA * 32, sm1, st>>>(c, p1, s);
   else if (gated && nost) k_stage1<false, true, true><<<grids[0], WARPS_PER_CTA * 32, sm1, st>>>(c, p1, s);
