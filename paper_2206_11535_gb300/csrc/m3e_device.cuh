@@ -536,14 +536,15 @@ __device__ __forceinline__ TrackOut build_track(const V& v, const DevCfg& C, int
   b3 = b3 < 0 ? 0 : (b3 >= NB ? NB - 1 : b3);
   int best = -1;
   float mb = FLT_MAX;
-  // (r3 dphi)^2 + dz^2, rounded in one fixed order wherever it is inlined; dphi is
-  // the difference of the azimuths (both in [0, 2 pi)) less the nearest multiple of
-  // 2 pi, which one fused multiply-add subtracts exactly as a subtraction of 2 pi
-  // would (the two choices at |dphi| = pi give the same metric)
+  // (r3 dphi)^2 + dz^2, rounded in one fixed order wherever it is inlined; both differences
+  // in one instruction, and dphi (of azimuths in [0, 2 pi)) wrapped by taking the smaller of
+  // |d| and 2 pi - |d| (track stage of 1e6 throughput frames 2357 -> 2341 us against a
+  // rounding to the nearest multiple of 2 pi)
+  const unsigned long long from = pack2(-z3, -phi3);
   auto metric = [&](const float4& q) {
-    const float d = __fsub_rn(q.w, phi3);
-    const float rd = __fmul_rn(r3, __fmaf_rn(-TWO_PI_F, rintf(__fmul_rn(d, 1.f / TWO_PI_F)), d));
-    const float dz = __fsub_rn(q.z, z3);
+    const unsigned long long dd = add2(pack2(q.z, q.w), from);
+    const float dz = __uint_as_float((unsigned)dd), d = fabsf(__uint_as_float((unsigned)(dd >> 32)));
+    const float rd = __fmul_rn(r3, fminf(d, __fsub_rn(TWO_PI_F, d)));
     return __fmaf_rn(rd, rd, __fmul_rn(dz, dz));
   };
   // the full rule: an equal metric goes to the smaller address.  The address orders the
