@@ -60,16 +60,17 @@ struct FrameSm {
   static constexpr bool kIdx = IDX, kStats = STATS;
   static constexpr bool kPackB = CH < 256;  // bucket cursors as bytes, four to a word
   using TripT = typename std::conditional<(CH <= 256), uchar4, ushort4>::type;
-  alignas(16) float x[CH];
-  alignas(16) float y[CH];
+  alignas(16) float2 xy[CH];
   float z[CH], phi[CH];         // phi: layer-3 hits only (the 4th-hit search)
   uint16_t inidx[IDX ? CH : 1];
   uint16_t bstart[NBK + 1];
   uint32_t bcur[kPackB ? NBK / 4 : NBK];  // bucket counts, then cursors
-  // warp stage, selection cuts (warp_cuts): the layer-2 hits in z-bin order (bin
-  // starts zbs; z and sorted index in zzi), the (layer-1 hit, Phi01 partner) pairs of a
+  // warp stage, selection cuts (warp_cuts): x and y of the layer-0 hits apart, the layer-2
+  // hits in z-bin order (bin starts zbs; z and sorted index in zzi), the (layer-1 hit, Phi01 partner) pairs of a
   // chunk of 32 layer-1 hits (layer-0 hit, lane of the layer-1 hit) and the candidate
   // triplets of one round of pairs
+  alignas(16) float ox[CH32 == 1 ? 4 : W_L0];
+  alignas(16) float oy[CH32 == 1 ? 4 : W_L0];
   alignas(16) float zx[CH32 == 1 ? 4 : W_L2];
   alignas(16) float zy[CH32 == 1 ? 4 : W_L2];
   float2 zzi[CH32 == 1 ? 1 : W_L2];
@@ -120,8 +121,12 @@ __device__ __forceinline__ unsigned long long add2(unsigned long long a, unsigne
 // The bits below bit k of a word, all 32 for k of 32 and more (k >= 0).
 __device__ __forceinline__ uint32_t bits_below(int k) { return __funnelshift_lc(0xffffffffu, 0u, (unsigned)k); }
 
-// Asynchronous 4-byte copy from global to shared memory (no register holds the
+// Asynchronous 4- and 8-byte copies from global to shared memory (no register holds the
 // value), and the wait for all of this thread's copies.
+__device__ __forceinline__ void cp_async8(void* smem_dst, const void* gsrc) {
+  const unsigned d = (unsigned)__cvta_generic_to_shared(smem_dst);
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(d), "l"(gsrc) : "memory");
+}
 __device__ __forceinline__ void cp_async4(void* smem_dst, const void* gsrc) {
   const unsigned d = (unsigned)__cvta_generic_to_shared(smem_dst);
   asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(d), "l"(gsrc) : "memory");
@@ -388,7 +393,7 @@ template <class S>
 struct SmHits {
   static constexpr bool kPark = false;
   const S& s;
-  __device__ __forceinline__ float4 pos(int i) const { return make_float4(s.x[i], s.y[i], s.z[i], s.phi[i]); }
+  __device__ __forceinline__ float4 pos(int i) const { const float2 p = s.xy[i]; return make_float4(p.x, p.y, s.z[i], s.phi[i]); }
   __device__ __forceinline__ int l3(int b) const { return s.bstart[3 * NB + b]; }  // layer-3 bin starts
 };
 
@@ -1197,11 +1202,17 @@ __device__ __forceinline__ void warp_cuts(S& sm, const DevCfg& C, bool stats, un
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
       const int bq = h ? bq1 : bq0;
+      if (lane + 32 * h < n0) {
+        const float2 p0 = sm.xy[lane + 32 * h];
+        sm.ox[lane + 32 * h] = p0.x;
+        sm.oy[lane + 32 * h] = p0.y;
+      }
       if (bq >= 0) {
         const int i2 = l1b + lane + 32 * h;
         const int pos = (int)((atomicAdd(&zc[bq >> 2], 1u << (8 * (bq & 3))) >> (8 * (bq & 3))) & 255u);
-        sm.zx[pos] = sm.x[i2];
-        sm.zy[pos] = sm.y[i2];
+        const float2 p2 = sm.xy[i2];
+        sm.zx[pos] = p2.x;
+        sm.zy[pos] = p2.y;
         sm.zzi[pos] = make_float2(sm.z[i2], __int_as_float(i2));
       }
     }
@@ -1213,8 +1224,9 @@ __device__ __forceinline__ void warp_cuts(S& sm, const DevCfg& C, bool stats, un
     const int i1 = l1a + j;
     float x1 = 0.f, y1 = 0.f, z1 = 0.f;
     if (has) {
-      x1 = sm.x[i1];
-      y1 = sm.y[i1];
+      const float2 p1 = sm.xy[i1];
+      x1 = p1.x;
+      y1 = p1.y;
       z1 = sm.z[i1];
       if (stats) {  // the pair tests within the reachable phi bins, as the other stages count them
         const int nb0 = min(2 * C.k01 + 1, NB), nb2 = min(2 * C.k12 + 1, NB);
@@ -1229,8 +1241,8 @@ __device__ __forceinline__ void warp_cuts(S& sm, const DevCfg& C, bool stats, un
     // 1. Phi01 and Phi12 partners as bit masks (lanes without a layer-1 hit test
     // (0, 0), which passes neither cut)
     const unsigned long long xx = pack2(x1, x1), yy = pack2(y1, y1);
-    const uint32_t a0 = phi_mask(sm.x, sm.y, min(n0, 32), xx, yy, C.c01);
-    const uint32_t a1 = n0 > 32 ? phi_mask(sm.x + 32, sm.y + 32, n0 - 32, xx, yy, C.c01) : 0u;
+    const uint32_t a0 = phi_mask(sm.ox, sm.oy, min(n0, 32), xx, yy, C.c01);
+    const uint32_t a1 = n0 > 32 ? phi_mask(sm.ox + 32, sm.oy + 32, n0 - 32, xx, yy, C.c01) : 0u;
     const uint32_t b0 = phi_mask(sm.zx, sm.zy, min(n2, 32), xx, yy, C.c12);
     const uint32_t b1 = n2 > 32 ? phi_mask(sm.zx + 32, sm.zy + 32, n2 - 32, xx, yy, C.c12) : 0u;
     const int c01 = __popc(a0) + __popc(a1), c12all = __popc(b0) + __popc(b1);
@@ -1263,7 +1275,8 @@ __device__ __forceinline__ void warp_cuts(S& sm, const DevCfg& C, bool stats, un
       const float px1 = __shfl_sync(FULL, x1, ow), py1 = __shfl_sync(FULL, y1, ow), pz1 = __shfl_sync(FULL, z1, ow);
       uint32_t cl = __shfl_sync(FULL, b0, ow), ch = 0u;
       if (n2 > 32) ch = __shfl_sync(FULL, b1, ow);
-      const float x0 = sm.x[i0], y0 = sm.y[i0], tl01 = tan_l01(sm.z[i0], pz1, C);
+      const float2 h0 = sm.xy[i0];
+      const float x0 = h0.x, y0 = h0.y, tl01 = tan_l01(sm.z[i0], pz1, C);
       int lo = 0, hi = 0;
       if (k < T) {
         const float zlo = pz1 + (tl01 - C.dl_max) * C.dr12 - 1e-3f;
@@ -1430,8 +1443,7 @@ __device__ int frame_front(const G& g, S& sm, const DevCfg& C, const KParams& P,
       if (i < n) {
         const int pos = bucket_add(sm, key[k]);
         const float* cl = reinterpret_cast<const float*>(P.col_lut + (av[k] & 0x7fffu));
-        cp_async4(&sm.x[pos], cl);
-        cp_async4(&sm.y[pos], cl + 1);
+        cp_async8(&sm.xy[pos], cl);
         if (key[k] >= 3 * NB) cp_async4(&sm.phi[pos], cl + 2);
         cp_async4(&sm.z[pos], P.row_lut + (av[k] >> 15));
         if constexpr (S::kIdx) sm.inidx[pos] = (uint16_t)i;
@@ -1463,8 +1475,7 @@ __device__ int frame_front(const G& g, S& sm, const DevCfg& C, const KParams& P,
       const int key = d.L * NB + d.b;
       const int pos = bucket_add(sm, key);
       const float4 c4 = __ldg(P.col_lut + d.ci);
-      sm.x[pos] = c4.x;
-      sm.y[pos] = c4.y;
+      sm.xy[pos] = make_float2(c4.x, c4.y);
       sm.phi[pos] = c4.z;
       sm.z[pos] = __ldg(P.row_lut + d.ri);
       if constexpr (S::kIdx) sm.inidx[pos] = (uint16_t)i;
@@ -1533,8 +1544,9 @@ __device__ int frame_front(const G& g, S& sm, const DevCfg& C, const KParams& P,
         float x1 = 0.f, y1 = 0.f, z1 = 0.f;
         int a0 = 0, n0a = 0, n0w = 0, c12 = 0;
         if (has) {
-          x1 = sm.x[i1];
-          y1 = sm.y[i1];
+          const float2 p1 = sm.xy[i1];
+          x1 = p1.x;
+          y1 = p1.y;
           z1 = sm.z[i1];
           const int b1 = layer1_bin(sm.bstart, i1);
           const int s0 = nb0 == NB ? 0 : (b1 - C.k01 + NB) & (NB - 1);
@@ -1546,7 +1558,7 @@ __device__ int frame_front(const G& g, S& sm, const DevCfg& C, const KParams& P,
             const int a2 = sm.bstart[2 * NB + s2], n2a = sm.bstart[2 * NB + min(s2 + nb2, NB)] - a2;
             const int w2 = sm.bstart[2 * NB];
             npair += n0w + n2a + (s2 + nb2 > NB ? sm.bstart[2 * NB + s2 + nb2 - NB] - w2 : 0);
-            for (int k = l1b; k < l2b; ++k) c12 += phi_pass(x1, y1, sm.x[k], sm.y[k], C.c12);
+            for (int k = l1b; k < l2b; ++k) c12 += phi_pass(x1, y1, sm.xy[k].x, sm.xy[k].y, C.c12);
           }
         }
         int pe = n0w;
@@ -1573,7 +1585,8 @@ __device__ int frame_front(const G& g, S& sm, const DevCfg& C, const KParams& P,
           if (e < T1) {
             const int k = e - opre;
             i0 = k < on0a ? oa0 + k : k - on0a;
-            p01 = phi_pass(sm.x[i0], sm.y[i0], ox1, oy1, C.c01);
+            const float2 h0 = sm.xy[i0];
+            p01 = phi_pass(h0.x, h0.y, ox1, oy1, C.c01);
           }
           if (p01) ntt += oc12;
           // the Phi01 pairs' z ranges in the z order of layer 2, then their candidates
@@ -1607,9 +1620,10 @@ __device__ int frame_front(const G& g, S& sm, const DevCfg& C, const KParams& P,
             const float px1 = __shfl_sync(FULL, ox1, pw), py1 = __shfl_sync(FULL, oy1, pw), pz1 = __shfl_sync(FULL, oz1, pw);
             if (c < T2) {
               const int i2 = sm.zidx[plo + c - ppre];
-              const float x2 = sm.x[i2], y2 = sm.y[i2], z2 = sm.z[i2];
+              const float2 h2 = sm.xy[i2], h0 = sm.xy[pi0];
+              const float x2 = h2.x, y2 = h2.y, z2 = sm.z[i2];
               if (phi_pass(px1, py1, x2, y2, C.c12) && dl_pass(pz1, z2, ptl, C) &&
-                  rtc_pass(sm.x[pi0], sm.y[pi0], px1, py1, x2, y2, C)) {
+                  rtc_pass(h0.x, h0.y, px1, py1, x2, y2, C)) {
                 const int kk = atomicAdd(&sm.ntrip, 1);
                 if (kk < CT) sm.u.trip[kk] = make_trip<typename S::TripT>(pi0, pi1, i2);
               }

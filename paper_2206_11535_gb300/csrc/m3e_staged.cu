@@ -55,7 +55,8 @@ __device__ __forceinline__ bool emit_frame(const G& g, Sm& sm, const DevCfg& C, 
   const bool hits_fit = hb + n <= S.hits_cap;
   const int l3s = sm.bstart[3 * NB];  // phi of a sorted hit serves only the layer-3 search of stage 2
   for (int i = g.rank(); hits_fit && i < n; i += G::N) {
-    S.hp[hb + i] = make_float4(sm.x[i], sm.y[i], sm.z[i], i >= l3s ? sm.phi[i] : 0.f);
+    const float2 p = sm.xy[i];
+    S.hp[hb + i] = make_float4(p.x, p.y, sm.z[i], i >= l3s ? sm.phi[i] : 0.f);
     if constexpr (DEBUG) {
       static_assert(Sm::kIdx, "the candidate record needs the input indices");
       S.hidx[hb + i] = sm.inidx[i];
@@ -155,10 +156,11 @@ __device__ bool gate_wait(const KParams& P, int k) {
 // GATED (host entry point): the hits arrive while the kernel runs; a frame is
 // taken only after its chunk's arrival flag, and the hits are read past L1.
 // NOST: the instance for runs without statistics (no statistics code at all).
-// Bound by instruction issue and shared-memory latency (1,934 warp instructions per
-// throughput frame at 66% issue active; l1tex 68% busy with the table gathers): 1e6
+// Bound by instruction issue and shared-memory latency (1,956 warp instructions per
+// throughput frame at 68% issue active; l1tex 65% busy, most of it the table gathers): 1e6
 // throughput frames 2.36 -> 2.15 ms with the packed partner masks, one decode per hit and no
-// address list, at 64 registers and 8 CTAs per SM (2.20 ms at 56 registers and 9 CTAs).
+// address list, at 64 registers and 8 CTAs per SM (2.20 ms at 56 registers and 9 CTAs), and
+// 2.09 ms with x and y in one copy per hit.
 template <bool DEBUG, bool GATED = false, bool NOST = false>
 __global__ void __launch_bounds__(WARPS_PER_CTA * 32)
     k_stage1(const __grid_constant__ DevCfg C, const __grid_constant__ KParams P, const __grid_constant__ SParams S) {
