@@ -216,7 +216,8 @@ template <bool GRAD>
 __global__ void __launch_bounds__(GT) k_fit_grad(const __grid_constant__ DevCfg C, const __grid_constant__ GradParams G) {
   __shared__ AlignSm A;
   static_assert(NG % 2 == 1, "odd row stride and 8 words between the warps: no bank conflicts");
-  __shared__ float red[GT / 32][32 * NG + 8];
+  __shared__ __align__(8) float red[GRAD ? GT / 32 : 1][GRAD ? 32 * NG + 8 : 4 * (GT / 32)];
+  pdl_trigger();
   if (threadIdx.x < 4) {
     const int L = threadIdx.x;
     float w[3] = {G.params[6 * L + 3], G.params[6 * L + 4], G.params[6 * L + 5]};
@@ -346,46 +347,58 @@ __global__ void __launch_bounds__(GT) k_fit_grad(const __grid_constant__ DevCfg 
     if (G.chi2_each) G.chi2_each[i] = ok ? chi2 : __int_as_float(0x7fc00000);
     if (G.kappa_each) G.kappa_each[i] = ok ? kb_out : __int_as_float(0x7fc00000);
   }
-  // block sums in FP64, fixed order: the threads' sums side by side in shared memory,
-  // then four threads per output, each adding 32 of them (8 times fewer FP64 additions,
-  // which are slow here, than a shuffle tree per output)
-  constexpr int KS[3] = {0, 25, 26};
+  // block sums in FP64, fixed order
   const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
   if (GRAD) {
+    // the threads' sums side by side in shared memory, then four threads per output, each
+    // adding 32 of them (8 times fewer FP64 additions, which are slow here, than a shuffle
+    // tree per output)
 #pragma unroll
     for (int k = 0; k < NG; ++k) red[wp][lane * NG + k] = acc[k];
-  } else {
-#pragma unroll
-    for (int k = 0; k < 3; ++k) red[wp][lane * NG + KS[k]] = acc[KS[k]];
-  }
-  __syncthreads();
-  const int k = threadIdx.x >> 2, part = threadIdx.x & 3;
-  double v = 0.0;
-  const bool used = k < NG && (GRAD || k == 0 || k == 26);
-  if (used) {
+    __syncthreads();
+    const int k = threadIdx.x >> 2, part = threadIdx.x & 3;
+    double v = 0.0;
+    if (k < NG) {
 #pragma unroll 8
-    for (int j = 0; j < 32; ++j) v += (double)red[part][j * NG + k];
+      for (int j = 0; j < 32; ++j) v += (double)red[part][j * NG + k];
+    }
+    v += __shfl_xor_sync(FULL, v, 1);
+    v += __shfl_xor_sync(FULL, v, 2);
+    if (k < NG && part == 0) G.partial[(int64_t)k * gridDim.x + blockIdx.x] = v;
+  } else {
+    double* const dred = reinterpret_cast<double*>(&red[0][0]);
+    double v = acc[0];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(FULL, v, o);
+    const unsigned nv = __reduce_add_sync(FULL, (unsigned)acc[26]);
+    if (lane == 0) {
+      dred[wp] = v;
+      dred[GT / 32 + wp] = (double)nv;
+    }
+    __syncthreads();
+    if (threadIdx.x < 2) {
+      double t = 0.0;
+      for (int k = 0; k < GT / 32; ++k) t += dred[threadIdx.x * (GT / 32) + k];
+      G.partial[(int64_t)(threadIdx.x ? 26 : 0) * gridDim.x + blockIdx.x] = t;
+    }
   }
-  v += __shfl_xor_sync(FULL, v, 1);
-  v += __shfl_xor_sync(FULL, v, 2);
-  if (used && part == 0) G.partial[(int64_t)k * gridDim.x + blockIdx.x] = v;
 }
 
 // Sum of the block partials: a warp per output, its lanes over the blocks, in a fixed
 // order; then the rotations' components from the moments.
 __global__ void __launch_bounds__(32 * NG)
-    k_fit_reduce(const double* __restrict__ partial, int nblocks, const float* __restrict__ params,
+    k_fit_reduce(const double* partial, int nblocks, const float* __restrict__ params,
                  unsigned long long* n_valid, float* chi2_sum, float* grad) {
   __shared__ double sum[NG];
-  const int k = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  if (k == 0 || k == 26 || grad) {
-    double v = 0.0;
-#pragma unroll 4
-    for (int b = lane; b < nblocks; b += 32) v += partial[(int64_t)k * nblocks + b];
+  // without the gradient two warps: the sum and the count
+  const int k = grad ? threadIdx.x >> 5 : (threadIdx.x >> 5) * (NG - 1), lane = threadIdx.x & 31;
+  pdl_wait();
+  double v = 0.0;
+#pragma unroll 16
+  for (int b = lane; b < nblocks; b += 32) v += __ldcg(partial + (int64_t)k * nblocks + b);
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(FULL, v, o);
-    if (lane == 0) sum[k] = v;
-  }
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(FULL, v, o);
+  if (lane == 0) sum[k] = v;
   __syncthreads();
   const int t = threadIdx.x;
   if (t == 31) *n_valid = (unsigned long long)sum[26];
@@ -448,8 +461,7 @@ cudaError_t launch_fit_grad(const DevCfg& c, const int32_t* hits, const int64_t*
   else k_fit_grad<false><<<nblocks, GT, 0, s>>>(c, g);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  k_fit_reduce<<<1, 32 * NG, 0, s>>>(partial, nblocks, params, n_valid, chi2_sum, grad);
-  return cudaGetLastError();
+  return launch_pdl(k_fit_reduce, 1, grad ? 32 * NG : 64, 0, s, (const double*)partial, nblocks, params, n_valid, chi2_sum, grad);
 }
 
 }  // namespace m3e
