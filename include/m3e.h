@@ -151,10 +151,11 @@ int m3e_destroy(m3e_ctx* ctx);
  * the throughput form: five persistent kernels that regroup the batch by
  * candidate (frames -> selected triplets -> tracks -> combinations -> decisions,
  * the candidates in device scratch); frames larger than a stage's capacity are
- * re-run by a CTA-per-frame kernel with identical decisions.  A batch of at most
- * 2048 frames without statistics or kernel timing runs a CTA per frame instead
- * (two launches, no scratch, the same decisions).  d_stats may be NULL.  n_frames
- * may be 0. */
+ * re-run by a CTA-per-frame kernel with identical decisions.  Without statistics
+ * or kernel timing a batch of at most 2048 frames runs a CTA per frame instead (two
+ * launches, no scratch), one of at most 8192 a single kernel that takes eight
+ * frames at a time through the method (the same decisions).  d_stats may be NULL.
+ * n_frames may be 0. */
 int m3e_select_frames(m3e_ctx* ctx, const int32_t* d_hits, const int64_t* d_frame_off, int64_t n_frames,
                       uint8_t* d_keep, uint8_t* d_reason, m3e_stats* d_stats, cudaStream_t stream);
 
@@ -282,8 +283,9 @@ int m3e_ingest(m3e_ctx* ctx, const int32_t* d_hits, int64_t n_hits, float* d_x, 
 
 /* Selection without any device allocation in the call (the paper has no
  * counterpart; this is a deployment aid).  Same decisions as m3e_select_frames,
- * through the fused kernels, with their scratch in a fixed static device array
- * instead of context memory that grows with the batch.  For callers that must
+ * through one persistent kernel that keeps every intermediate in shared memory,
+ * with its queue and deferred list in a fixed static device array instead of
+ * context memory that grows with the batch.  For callers that must
  * not allocate once running: a filter loop at a fixed frame rate cannot take the
  * device synchronisation of cudaMalloc/cudaFree, and a process sharing the GPU
  * under a fixed memory budget reserves all memory at start-up.  The context must
@@ -294,8 +296,8 @@ int m3e_ingest(m3e_ctx* ctx, const int32_t* d_hits, int64_t n_hits, float* d_x, 
  *     make that first call before any stream capture.  The address is cached per
  *     device; m3e_create clears the cache, so after a cudaDeviceReset create a
  *     new context before calling again.
- *   - Frames above the context's warp-tier size (set by m3e_autotune)
- *     go to the CTA-per-frame kernel, as in m3e_select_frames_fused.
+ *   - Frames above the context's warp-tier size (set by m3e_autotune) go to
+ *     CTA-per-frame kernels.
  *   - The array is shared by all calls on a device and keeps the last call's
  *     contents; the call clears what must start at zero.  Calls that overlap on
  *     the GPU (other streams, other contexts of the same device, other threads)

@@ -91,7 +91,7 @@ struct Scratch {
 struct m3e_ctx {
   int device = 0;
   int sms = 1;
-  int fused_bpsm = 1, s1_bpsm = 1, s2_bpsm = 1, s3_bpsm = 1, s4_bpsm = 1, s1c_bpsm = 1, s1m_bpsm = 1, ingest_bpsm = 1;
+  int fused_bpsm = 1, group_bpsm = 1, s1_bpsm = 1, s2_bpsm = 1, s3_bpsm = 1, s4_bpsm = 1, s1c_bpsm = 1, s1m_bpsm = 1, ingest_bpsm = 1;
   int grab = 4;
   int defer_hits = W_HITS;
   int mid_threads = CTA_THREADS;  // threads of a stage-1 middle-tier CTA
@@ -388,23 +388,36 @@ int check_batch(const int32_t* hits, const int64_t* off, int64_t n, const uint8_
 
 enum { FORM_STAGED = 0, FORM_FUSED = 1, FORM_PLAIN = 2 };
 
-// Whether a call that asks for the staged form takes a CTA per frame instead (the same
-// decisions): a small batch of a decision-only run, for which two launches and one frame's
-// latency replace eight launches and two memsets.
-bool takes_small(int form, int64_t n, bool debug, bool timed, const void* stats) {
-  return form == FORM_STAGED && n <= SMALL_FRAMES && !debug && !timed && !stats;
+// What a call that asks for the staged form takes (the same decisions): a decision-only run
+// of a small batch a CTA per frame, of a middle-sized one the group form; these save most of
+// the staged form's eight launches and their tails.
+enum Route { ROUTE_FORM, ROUTE_SMALL, ROUTE_GROUP };
+Route route_of(int form, int64_t n, bool debug, bool timed, const void* stats) {
+  if (form != FORM_STAGED || n > GROUP_FRAMES || debug || timed || stats) return ROUTE_FORM;
+  return n <= SMALL_FRAMES ? ROUTE_SMALL : ROUTE_GROUP;
 }
 
-// Enqueue one batch on stream s: form 0 staged (5 kernels; small batches a CTA per frame
-// unless `small` is false), 1 fused warp kernel, 2 plain CTA-per-frame kernel; forms 0 and
+// One decision-only batch in the group form: p.work and the deferred list are its only scratch.
+int enqueue_group(m3e_ctx* x, const KParams& p, cudaStream_t s) {
+  CUDA_TRY(cudaMemsetAsync(p.work, 0, 2 * sizeof(int), s));  // queue head and deferred count
+  CUDA_TRY(launch_group(x->dc, p, x->sms * x->group_bpsm, s));
+  CUDA_TRY(launch_deferred(x->dc, p, 2 * x->sms, false, s, true));
+  x->last_launches = 2;
+  return M3E_OK;
+}
+
+// Enqueue one batch on stream s: form 0 staged (5 kernels; smaller batches as route_of says
+// unless `reroute` is false), 1 fused warp kernel, 2 plain CTA-per-frame kernel; forms 0 and
 // 1 finish with the deferred-frame kernel.  Timing events are recorded when `timed`.
 int enqueue(m3e_ctx* x, Scratch& sc, KParams p, int form, bool debug, cudaStream_t s, bool timed,
-            cudaEvent_t after_s1 = nullptr, bool small = true) {
-  if (small && !p.gate && takes_small(form, p.n_frames, debug, timed, p.stats)) {
+            cudaEvent_t after_s1 = nullptr, bool reroute = true) {
+  const Route route = reroute && !p.gate ? route_of(form, p.n_frames, debug, timed, p.stats) : ROUTE_FORM;
+  if (route == ROUTE_SMALL) {
     CUDA_TRY(launch_small(x->dc, p, x->sms, s));
     x->last_launches = 2;
     return M3E_OK;
   }
+  if (route == ROUTE_GROUP) return enqueue_group(x, p, s);
   // frames per queue grab: at least two grabs for every resident warp, so that a batch of
   // a few frames per warp spreads over all of them
   const int64_t warps = (int64_t)x->sms * WARPS_PER_CTA * (form == FORM_FUSED ? x->fused_bpsm : x->s1_bpsm);
@@ -421,7 +434,7 @@ int enqueue(m3e_ctx* x, Scratch& sc, KParams p, int form, bool debug, cudaStream
     if (timed) CUDA_TRY(cudaEventRecord(x->pe[0], s));
     CUDA_TRY(launch_fused(x->dc, p, x->sms * x->fused_bpsm, debug, s));
     if (timed) CUDA_TRY(cudaEventRecord(x->pe[1], s));
-    CUDA_TRY(launch_deferred(x->dc, p, 2 * x->sms, debug, s));
+    CUDA_TRY(launch_deferred(x->dc, p, 2 * x->sms, debug, s, !timed));
     if (timed) CUDA_TRY(cudaEventRecord(x->pe[2], s));
     x->last_launches = 2;
     return M3E_OK;
@@ -435,7 +448,7 @@ int enqueue(m3e_ctx* x, Scratch& sc, KParams p, int form, bool debug, cudaStream
   KParams pd = p;  // frames no stage could finish: the CTA-per-frame kernel
   pd.in_list = sp.list2;
   pd.in_count = sp.lcount + 1;
-  CUDA_TRY(launch_deferred(x->dc, pd, 2 * x->sms, debug, s));
+  CUDA_TRY(launch_deferred(x->dc, pd, 2 * x->sms, debug, s, !timed && p.n_frames <= DEPENDENT_FRAMES));
   if (timed) CUDA_TRY(cudaEventRecord(x->pe[8], s));
   x->last_launches = 8;
   return M3E_OK;
@@ -471,6 +484,7 @@ int m3e_create(const m3e_config* cfg, int cuda_device, m3e_ctx** out) {
   }
   x->sms = prop.multiProcessorCount;
   x->fused_bpsm = fused_blocks_per_sm();
+  x->group_bpsm = group_blocks_per_sm();
   x->s1_bpsm = stage_blocks_per_sm(1);
   x->s2_bpsm = stage_blocks_per_sm(2);
   x->s3_bpsm = stage_blocks_per_sm(3);
@@ -601,7 +615,8 @@ static int select_common(m3e_ctx* x, const int32_t* hits, const int64_t* off, in
   if (n == 0) return M3E_OK;
   DeviceGuard guard(x->device);
   const bool timed = x->prof && dump == nullptr;
-  if (!takes_small(form, n, dump != nullptr, timed, stats)) rc = ensure_scratch(x->main, n, form == FORM_STAGED);
+  const Route route = route_of(form, n, dump != nullptr, timed, stats);
+  if (route != ROUTE_SMALL) rc = ensure_scratch(x->main, n, form == FORM_STAGED && route == ROUTE_FORM);
   if (rc) return rc;
   KParams p = base_params(x, x->main);
   p.hits = hits;
@@ -790,7 +805,7 @@ extern "C" int m3e_ingest(m3e_ctx* x, const int32_t* d_hits, int64_t n_hits, flo
 
 // ------------------------------------------------------------------ selection without allocation
 //
-// m3e_select_frames_noalloc runs the fused kernels with their scratch (work-queue
+// m3e_select_frames_noalloc runs the group form with its scratch (work-queue
 // head, deferred-frame count, deferred-frame list) in the static device array
 // below instead of context memory that grows with the batch.  It exists for
 // callers that must not allocate device memory once they are running: a filter
@@ -878,12 +893,7 @@ extern "C" int m3e_select_frames_noalloc(m3e_ctx* x, const int32_t* d_hits, cons
   p.n_frames = n_frames;
   p.keep = d_keep;
   p.reason = d_reason;
-  // the queue head and the deferred count start at zero; the list is written before it is read
-  CUDA_TRY(cudaMemsetAsync(scratch, 0, 2 * sizeof(int), s));
-  CUDA_TRY(launch_fused(x->dc, p, x->sms * x->fused_bpsm, false, s));
-  CUDA_TRY(launch_deferred(x->dc, p, 2 * x->sms, false, s));
-  x->last_launches = 2;
-  return M3E_OK;
+  return enqueue_group(x, p, s);
 }
 
 // ------------------------------------------------------------------ persistent batched form

@@ -133,7 +133,7 @@ __device__ __forceinline__ void cp_async4(void* smem_dst, const void* gsrc) {
 }
 // Programmatic dependent launch.  pdl_wait: wait until the preceding kernel of the stream
 // has finished and its writes are visible (nothing to wait for in an ordinary launch);
-// every block of a kernel launched with launch_pdl calls it before it reads or writes
+// every block of a kernel launched as a dependent calls it before it reads or writes
 // memory.  pdl_trigger: the following kernel's blocks may be placed once every block of
 // this one has got here or ended.
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
@@ -1806,10 +1806,10 @@ __device__ __forceinline__ void clear_stats(const G& g, S& sm) {
   g.sync();
 }
 
-// Launch with programmatic stream serialisation: the launch and the prologue overlap the
-// end of the kernel before it on the stream.
+// Launch, with pdl as a programmatic dependent of the kernel before it on the stream: the
+// launch and the prologue overlap that kernel's end.
 template <class... K, class... A>
-cudaError_t launch_pdl(void (*k)(K...), int grid, int threads, size_t smem, cudaStream_t s, const A&... a) {
+cudaError_t launch_kernel(bool pdl, void (*k)(K...), int grid, int threads, size_t smem, cudaStream_t s, const A&... a) {
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3((unsigned)grid);
   cfg.blockDim = dim3((unsigned)threads);
@@ -1819,7 +1819,7 @@ cudaError_t launch_pdl(void (*k)(K...), int grid, int threads, size_t smem, cuda
   at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
   at.val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = &at;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = pdl ? 1 : 0;
   return cudaLaunchKernelEx(&cfg, k, a...);
 }
 

@@ -55,6 +55,7 @@ __global__ void __launch_bounds__(NT) k_select_cta(const __grid_constant__ DevCf
   SmCta& sm = *reinterpret_cast<SmCta*>(smem_raw);
   const CtaGroup<NT> g;
   clear_stats(g, sm);
+  if (LIST) pdl_wait();
   const int count = LIST ? *P.in_count : (int)P.n_frames;
   for (int i = blockIdx.x; i < count; i += gridDim.x) {
     const int f = LIST ? P.in_list[i] : i;
@@ -69,7 +70,8 @@ __global__ void __launch_bounds__(NT) k_select_cta(const __grid_constant__ DevCf
 // Small batches: a CTA per frame with a stage of 512 hits, so that a whole small batch is
 // resident at once and the call takes one frame's latency.  A frame beyond the stage is
 // marked in its reason for k_select_marked.
-using SmSmall = FrameSm<SMALL_HITS, SMALL_TRIP, C_TRK, C_COMBO>;
+using SmSmall = FrameSm<SMALL_HITS, SMALL_TRIP, C_TRK, C_COMBO, false, false>;
+static_assert(8 * (sizeof(SmSmall) + 1024) <= 228 * 1024, "eight CTAs per SM");
 constexpr uint8_t MARK = 0xff;
 
 // NT: threads of a CTA, CTAS: of them per SM.  Measured (us, batches of nominal / throughput /
@@ -150,16 +152,19 @@ cudaError_t launch_fused(const DevCfg& c, const KParams& p, int grid, bool debug
   return cudaGetLastError();
 }
 
-cudaError_t launch_deferred(const DevCfg& c, const KParams& p, int grid, bool debug, cudaStream_t s) {
+// pdl: the kernel before it on the stream is the one that wrote the list.
+cudaError_t launch_deferred(const DevCfg& c, const KParams& p, int grid, bool debug, cudaStream_t s, bool pdl) {
   const size_t sm = cta_smem_bytes();
   if (debug) {
     cudaError_t e = set_smem(k_select_cta<CTA_THREADS, true, true>, sm);
     if (e != cudaSuccess) return e;
-    k_select_cta<CTA_THREADS, true, true><<<grid, CTA_THREADS, sm, s>>>(c, p);
+    e = launch_kernel(pdl, k_select_cta<CTA_THREADS, true, true>, grid, CTA_THREADS, sm, s, c, p);
+    if (e != cudaSuccess) return e;
   } else {
     cudaError_t e = set_smem(k_select_cta<CTA_THREADS, false, true>, sm);
     if (e != cudaSuccess) return e;
-    k_select_cta<CTA_THREADS, false, true><<<grid, CTA_THREADS, sm, s>>>(c, p);
+    e = launch_kernel(pdl, k_select_cta<CTA_THREADS, false, true>, grid, CTA_THREADS, sm, s, c, p);
+    if (e != cudaSuccess) return e;
   }
   return cudaGetLastError();
 }
@@ -174,7 +179,7 @@ cudaError_t launch_small(const DevCfg& c, KParams p, int sms, cudaStream_t s) {
   if (wide) k_select_small<256, 4><<<(int)p.n_frames, 256, sizeof(SmSmall), s>>>(c, p);
   else k_select_small<128, 8><<<(int)p.n_frames, 128, sizeof(SmSmall), s>>>(c, p);
   const int grid = (int)(p.n_frames < 2 * sms ? p.n_frames : 2 * sms);
-  return launch_pdl(k_select_marked, grid, CTA_THREADS, sizeof(SmCta), s, c, p);
+  return launch_kernel(true, k_select_marked, grid, CTA_THREADS, sizeof(SmCta), s, c, p);
 }
 
 cudaError_t launch_plain(const DevCfg& c, const KParams& p, bool debug, cudaStream_t s) {

@@ -461,7 +461,7 @@ cudaError_t launch_fit_grad(const DevCfg& c, const int32_t* hits, const int64_t*
   else k_fit_grad<false><<<nblocks, GT, 0, s>>>(c, g);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  return launch_pdl(k_fit_reduce, 1, grad ? 32 * NG : 64, 0, s, (const double*)partial, nblocks, params, n_valid, chi2_sum, grad);
+  return launch_kernel(true, k_fit_reduce, 1, grad ? 32 * NG : 64, 0, s, (const double*)partial, nblocks, params, n_valid, chi2_sum, grad);
 }
 
 }  // namespace m3e

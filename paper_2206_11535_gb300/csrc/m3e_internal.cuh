@@ -31,6 +31,16 @@ constexpr int PLAIN_THREADS = 128;  // plain per-frame kernel
 // earlier (1000 frames 263 and 256, 2048 430 and 345).
 constexpr int SMALL_HITS = 512, SMALL_TRIP = 512;
 constexpr int64_t SMALL_FRAMES = 2048;
+// Middle-sized batches: the group form.  Up to how many frames: against the staged form 4096
+// and 8192 nominal frames take 27 and 42 us (49 and 60), parity frames 32 and 48 (53 and 66),
+// throughput frames 72 and 105 (81 and 117), 32-track frames 128 and 207 (136 and 189), uneven
+// ones 144 and 231 (155 and 204), 64-track frames 460 and 851 (332 and 579); 32,768 nominal
+// ones 130 (113).  The line favours the usual rates.
+constexpr int64_t GROUP_FRAMES = 8192;
+// Batches of the staged form whose kernels are launched as dependents of each other: the
+// waiting CTAs hide the launches (16,384 nominal frames 94 -> 80 us) but hold slots that the
+// persistent kernels of a large batch need (131,072 throughput frames 833 -> 867 us).
+constexpr int64_t DEPENDENT_FRAMES = 16384;
 
 // Geometry and cuts, precomputed on the host in FP64 and rounded once.
 struct DevCfg {
@@ -115,11 +125,13 @@ enum { ERR_BADHIT = 1, ERR_NEGSIZE = 2, ERR_GATE = 4 };
 
 // Host-side launchers (m3e_fused.cu, m3e_staged.cu).
 cudaError_t launch_fused(const DevCfg& c, const KParams& p, int grid, bool debug, cudaStream_t s);
-cudaError_t launch_deferred(const DevCfg& c, const KParams& p, int grid, bool debug, cudaStream_t s);
+cudaError_t launch_deferred(const DevCfg& c, const KParams& p, int grid, bool debug, cudaStream_t s, bool pdl);
 cudaError_t launch_small(const DevCfg& c, KParams p, int sms, cudaStream_t s);
 cudaError_t launch_plain(const DevCfg& c, const KParams& p, bool debug, cudaStream_t s);
 cudaError_t launch_staged(const DevCfg& c, const KParams& p, const SParams& s, const int grids[6], bool debug,
                           cudaStream_t st, cudaEvent_t* ev, cudaEvent_t after_s1 = nullptr, int mid_threads = 256);
+cudaError_t launch_group(const DevCfg& c, const KParams& p, int resident, cudaStream_t s);
+int group_blocks_per_sm();
 int stage1_mid_blocks_per_sm(int threads);  // resident CTAs per SM of the stage-1 middle tier
 size_t stage1c_smem_bytes();
 int fused_blocks_per_sm();
