@@ -170,6 +170,7 @@ __global__ void __launch_bounds__(WARPS_PER_CTA * 32)
   __shared__ long long bcast[WARPS_PER_CTA][2];
   const WarpGroup g;
   if (!NOST) clear_stats(g, sm);
+  pdl_trigger();
   const int nf = (int)P.n_frames;
   int arrived = -1;  // chunks up to this one are known to have arrived
   bool stop = false;
@@ -208,6 +209,8 @@ __global__ void __launch_bounds__(NT)
   __shared__ long long bcast[2];
   const CtaGroup<NT> g;
   clear_stats(g, sm);
+  pdl_trigger();
+  pdl_wait();
   const int count = *P.in_count;
   for (int i = blockIdx.x; i < count; i += gridDim.x) {
     const int f = P.in_list[i];
@@ -225,6 +228,8 @@ __global__ void __launch_bounds__(128, 8)  // 8 CTAs per SM (64 registers: the f
     k_stage2(const __grid_constant__ DevCfg C, const __grid_constant__ KParams P, const __grid_constant__ SParams S) {
   static_assert(sizeof(FitPark) == 11 * 128 * sizeof(float), "one slot per thread of a 128-thread CTA");
   __shared__ FitPark park;
+  pdl_trigger();
+  pdl_wait();
   const int64_t n = min((int64_t)S.counters[0], S.trip_cap);
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
@@ -288,6 +293,8 @@ __global__ void __launch_bounds__(S3_WARPS * 32, 10)
   if (!NOST)
     for (int k = lane; k < ST_REASON0 + 8; k += 32) sm.acc[k] = 0;
   __syncwarp();
+  pdl_trigger();
+  pdl_wait();
   const int nf = (int)P.n_frames;
   const bool stats = !NOST && P.stats != nullptr;
   // all energy-test survivors count towards the cap; a decision-only run writes only those
@@ -481,6 +488,8 @@ __global__ void __launch_bounds__(S4_WARPS * 32, 8)  // 8 CTAs per SM (64 regist
   __shared__ long long queue[S4_WARPS][64];
   long long* q = queue[threadIdx.x >> 5];
   const int lane = threadIdx.x & 31;
+  pdl_trigger();
+  pdl_wait();
   const int64_t n = min((int64_t)S.counters[1], S.combo_cap);
   const int64_t stride = (int64_t)gridDim.x * S4_WARPS * 32;
   int qn = 0;
@@ -546,6 +555,8 @@ __global__ void __launch_bounds__(256)
     k_stage5(const __grid_constant__ KParams P, const __grid_constant__ SParams S) {
   __shared__ unsigned cnt[2];
   if (threadIdx.x < 2) cnt[threadIdx.x] = 0;
+  pdl_trigger();
+  pdl_wait();
   __syncthreads();
   const int f = blockIdx.x * blockDim.x + threadIdx.x;
   if (f < P.n_frames && S.fstate[f] == PENDING) {
@@ -617,24 +628,25 @@ int stage1_mid_blocks_per_sm(int threads) {
 // null): before stage 1 and after each kernel.
 // One launch of a CTA tier of stage 1 (the instance without statistics code when nost).
 template <class Sm, int CH, bool DEBUG, int NT>
-cudaError_t launch_tier(const DevCfg& c, const KParams& p, const SParams& s, int grid, size_t smem, cudaStream_t st,
-                        bool nost) {
+cudaError_t launch_tier(bool pdl, const DevCfg& c, const KParams& p, const SParams& s, int grid, size_t smem,
+                        cudaStream_t st, bool nost) {
   if constexpr (!DEBUG) {
     if (nost) {
       const cudaError_t e = set_smem(k_stage1c<Sm, CH, false, NT, true>, smem);
-      if (e == cudaSuccess) k_stage1c<Sm, CH, false, NT, true><<<grid, NT, smem, st>>>(c, p, s);
-      return e;
+      return e != cudaSuccess ? e : launch_kernel(pdl, k_stage1c<Sm, CH, false, NT, true>, grid, NT, smem, st, c, p, s);
     }
   }
   const cudaError_t e = set_smem(k_stage1c<Sm, CH, DEBUG, NT>, smem);
-  if (e == cudaSuccess) k_stage1c<Sm, CH, DEBUG, NT><<<grid, NT, smem, st>>>(c, p, s);
-  return e;
+  return e != cudaSuccess ? e : launch_kernel(pdl, k_stage1c<Sm, CH, DEBUG, NT>, grid, NT, smem, st, c, p, s);
 }
 
 cudaError_t launch_staged(const DevCfg& c, const KParams& p, const SParams& s, const int grids[6], bool debug,
                           cudaStream_t st, cudaEvent_t* ev, cudaEvent_t after_s1, int mid_threads) {
   const bool gated = p.gate != nullptr && !debug;
   const bool nost = p.stats == nullptr;
+  // every kernel after the first a programmatic dependent of the one before it, unless each
+  // is timed apart or a copy stream's event comes between
+  const bool pdl = ev == nullptr && p.n_frames <= DEPENDENT_FRAMES;
   const size_t sm1 = stage1_smem_bytes(debug, nost), smc = stage1c_smem_bytes(), smm = stage1m_smem_bytes();
   cudaError_t e = debug ? set_smem(k_stage1<true>, sm1)
                   : gated ? (nost ? set_smem(k_stage1<false, true, true>, sm1) : set_smem(k_stage1<false, true>, sm1))
@@ -664,29 +676,32 @@ cudaError_t launch_staged(const DevCfg& c, const KParams& p, const SParams& s, c
   // the later kernels read the hits too: order them after every copy of the host entry
   if (after_s1) cudaStreamWaitEvent(st, after_s1, 0);
   if (ev) cudaEventRecord(ev[1], st);
-  e = debug ? launch_tier<SmFrontMid, M_HITS, true, CTA_THREADS>(c, pm, s, grids[5], smm, st, false)
-            : mid_threads == 128 ? launch_tier<SmFrontMid, M_HITS, false, 128>(c, pm, s, grids[5], smm, st, nost)
-            : mid_threads == 512 ? launch_tier<SmFrontMid, M_HITS, false, 512>(c, pm, s, grids[5], smm, st, nost)
-                                 : launch_tier<SmFrontMid, M_HITS, false, CTA_THREADS>(c, pm, s, grids[5], smm, st, nost);
+  e = debug ? launch_tier<SmFrontMid, M_HITS, true, CTA_THREADS>(pdl && !after_s1, c, pm, s, grids[5], smm, st, false)
+            : mid_threads == 128 ? launch_tier<SmFrontMid, M_HITS, false, 128>(pdl && !after_s1, c, pm, s, grids[5], smm, st, nost)
+            : mid_threads == 512 ? launch_tier<SmFrontMid, M_HITS, false, 512>(pdl && !after_s1, c, pm, s, grids[5], smm, st, nost)
+                                 : launch_tier<SmFrontMid, M_HITS, false, CTA_THREADS>(pdl && !after_s1, c, pm, s, grids[5], smm, st, nost);
   if (e != cudaSuccess) return e;
   if (ev) cudaEventRecord(ev[2], st);
-  e = debug ? launch_tier<SmFrontCta, C_HITS, true, CTA_THREADS>(c, pc, s, grids[4], smc, st, false)
-            : launch_tier<SmFrontCta, C_HITS, false, CTA_THREADS>(c, pc, s, grids[4], smc, st, nost);
+  e = debug ? launch_tier<SmFrontCta, C_HITS, true, CTA_THREADS>(pdl, c, pc, s, grids[4], smc, st, false)
+            : launch_tier<SmFrontCta, C_HITS, false, CTA_THREADS>(pdl, c, pc, s, grids[4], smc, st, nost);
   if (e != cudaSuccess) return e;
   if (ev) cudaEventRecord(ev[3], st);
-  if (debug) k_stage2<true><<<grids[1], 128, 0, st>>>(c, p, s);
-  else k_stage2<false><<<grids[1], 128, 0, st>>>(c, p, s);
+  const auto go = [&](auto k, int grid, int threads, const auto&... args) {
+    if (e == cudaSuccess) e = launch_kernel(pdl, k, grid, threads, 0, st, args...);
+  };
+  if (debug) go(k_stage2<true>, grids[1], 128, c, p, s);
+  else go(k_stage2<false>, grids[1], 128, c, p, s);
   if (ev) cudaEventRecord(ev[4], st);
-  if (debug) k_stage3<true><<<grids[2], S3_WARPS * 32, 0, st>>>(c, p3, s);
-  else if (nost) k_stage3<false, true><<<grids[2], S3_WARPS * 32, 0, st>>>(c, p3, s);
-  else k_stage3<false><<<grids[2], S3_WARPS * 32, 0, st>>>(c, p3, s);
+  if (debug) go(k_stage3<true>, grids[2], S3_WARPS * 32, c, p3, s);
+  else if (nost) go(k_stage3<false, true>, grids[2], S3_WARPS * 32, c, p3, s);
+  else go(k_stage3<false>, grids[2], S3_WARPS * 32, c, p3, s);
   if (ev) cudaEventRecord(ev[5], st);
-  if (debug) k_stage4<true><<<grids[3], S4_WARPS * 32, 0, st>>>(c, p, s);
-  else if (nost) k_stage4<false, true><<<grids[3], S4_WARPS * 32, 0, st>>>(c, p, s);
-  else k_stage4<false><<<grids[3], S4_WARPS * 32, 0, st>>>(c, p, s);
+  if (debug) go(k_stage4<true>, grids[3], S4_WARPS * 32, c, p, s);
+  else if (nost) go(k_stage4<false, true>, grids[3], S4_WARPS * 32, c, p, s);
+  else go(k_stage4<false>, grids[3], S4_WARPS * 32, c, p, s);
   if (ev) cudaEventRecord(ev[6], st);
-  const int g5 = (int)((p.n_frames + 255) / 256);
-  if (g5 > 0) k_stage5<<<g5, 256, 0, st>>>(p, s);
+  go(k_stage5, (int)((p.n_frames + 255) / 256), 256, p, s);
+  if (e != cudaSuccess) return e;
   if (ev) cudaEventRecord(ev[7], st);
   return cudaGetLastError();
 }
