@@ -91,7 +91,7 @@ struct Scratch {
 struct m3e_ctx {
   int device = 0;
   int sms = 1;
-  int fused_bpsm = 1, group_bpsm = 1, s1_bpsm = 1, s2_bpsm = 1, s3_bpsm = 1, s4_bpsm = 1, s1c_bpsm = 1, s1m_bpsm = 1, ingest_bpsm = 1;
+  int fused_bpsm = 1, group_bpsm = 1, s1_bpsm = 1, s2_bpsm = 1, s3_bpsm = 1, s4_bpsm = 1, s1c_bpsm = 1, s1m_bpsm = 1;
   int grab = 4;
   int defer_hits = W_HITS;
   int mid_threads = CTA_THREADS;  // threads of a stage-1 middle-tier CTA
@@ -491,7 +491,6 @@ int m3e_create(const m3e_config* cfg, int cuda_device, m3e_ctx** out) {
   x->s4_bpsm = stage_blocks_per_sm(4);
   x->s1c_bpsm = stage_blocks_per_sm(5);
   x->s1m_bpsm = stage_blocks_per_sm(6);
-  x->ingest_bpsm = ingest_blocks_per_sm();
   x->fit_bpsm = fit_grad_blocks_per_sm(false);
   x->fit_grad_bpsm = fit_grad_blocks_per_sm(true);
   // look-up tables in FP64, rounded once
@@ -798,7 +797,7 @@ extern "C" int m3e_ingest(m3e_ctx* x, const int32_t* d_hits, int64_t n_hits, flo
   if (!d_hits || !d_x || !d_y || !d_z) return fail(M3E_EINVAL, "NULL hit or coordinate array");
   DeviceGuard guard(x->device);
   CUDA_TRY(launch_ingest(x->dc, d_hits, n_hits, x->col_lut, x->row_lut, d_x, d_y, d_z, d_phi, x->err,
-                         x->sms * x->ingest_bpsm, s));
+                         x->sms, s));
   x->last_launches = 1;
   return M3E_OK;
 }
