@@ -82,6 +82,7 @@ struct FrameSm {
   uint16_t zidx[CH32 == 1 ? CH : 1];
   uint16_t zbs2[CH32 == 1 ? NZB + 1 : 1];
   uint32_t zcur[CH32 == 1 ? NZB : 1];
+  uint8_t own[CH32 == 1 ? 16 : 1][2][32];  // per warp: the lanes that have window entries / candidates, in order
   TrkSoA<CK> t;                 // positives from the front, negatives from the back
   union {
     TripT trip[CT];             // selected triplets (sorted-hit indices)
@@ -1497,10 +1498,8 @@ __device__ int frame_front(const G& g, S& sm, const DevCfg& C, const KParams& P,
       // lambda cut of a (layer-0, layer-1) pair, seen as a z window on the layer-2 hit
       // (widened by 1e-3 mm against rounding), is one contiguous range of that order.
       // Each warp holds 32 layer-1 hits at a time and tests the entries of their Phi01
-      // windows 32 at a time (each lane finds its hit by a search over the lanes'
-      // prefix of window sizes); the z ranges of the pairs that pass are numbered by a
-      // prefix sum, and their candidates are tested 32 at a time (a second search)
-      // with the exact Phi12, Delta lambda and r_tc expressions of the warp stage.  The z window holds every hit that
+      // windows 32 at a time; the z ranges of the pairs that pass are numbered by a
+      // prefix sum, and their candidates are tested 32 at a time with the exact Phi12, Delta lambda and r_tc expressions of the warp stage.  The z window holds every hit that
       // passes Delta lambda, so the selected set equals the brute-force one.  A frame
       // whose triplet count passed max_trip overflows whatever follows: the warps stop.
       constexpr int NW = G::N / 32;
@@ -1568,14 +1567,21 @@ __device__ int frame_front(const G& g, S& sm, const DevCfg& C, const KParams& P,
           if (lane >= o) pe += t;
         }
         const int pre1 = pe - n0w, T1 = __shfl_sync(FULL, pe, 31);
+        // Which lane owns entry e: the lanes with entries are listed in order; the starts that
+        // fall on these 32 entries are or-ed into a word, and the starts up to e counted.
+        const unsigned upto = 0xffffffffu >> (31 - lane);
+        uint8_t* const own1 = sm.own[wid][0];
+        uint8_t* const own2 = sm.own[wid][1];
+        const unsigned ne1 = __ballot_sync(FULL, n0w > 0);
+        __syncwarp();
+        if (n0w > 0) own1[__popc(ne1 & upto) - 1] = (uint8_t)lane;
+        __syncwarp();
+        int before1 = -1;  // starts before these entries, less one
         for (int e0 = 0; e0 < T1 && !stop; e0 += 32) {
           const int e = e0 + lane;
-          int ow = 0;  // the last lane whose window entries start at or before e
-#pragma unroll
-          for (int st = 16; st; st >>= 1) {
-            const int pv = __shfl_sync(FULL, pre1, ow + st);
-            if (pv <= e) ow += st;
-          }
+          const unsigned s1 = __reduce_or_sync(FULL, n0w > 0 && (unsigned)(pre1 - e0) < 32u ? 1u << (pre1 - e0) : 0u);
+          const int ow = own1[before1 + __popc(s1 & upto)];
+          before1 += __popc(s1);
           const int oa0 = __shfl_sync(FULL, a0, ow), on0a = __shfl_sync(FULL, n0a, ow);
           const int opre = __shfl_sync(FULL, pre1, ow), oi1 = __shfl_sync(FULL, i1, ow);
           const float ox1 = __shfl_sync(FULL, x1, ow), oy1 = __shfl_sync(FULL, y1, ow), oz1 = __shfl_sync(FULL, z1, ow);
@@ -1606,14 +1612,16 @@ __device__ int frame_front(const G& g, S& sm, const DevCfg& C, const KParams& P,
             if (lane >= o) ce += t;
           }
           const int pre2 = ce - cnt, T2 = __shfl_sync(FULL, ce, 31);
+          const unsigned ne2 = __ballot_sync(FULL, cnt > 0);
+          __syncwarp();
+          if (cnt > 0) own2[__popc(ne2 & upto) - 1] = (uint8_t)lane;
+          __syncwarp();
+          int before2 = -1;
           for (int c0 = 0; c0 < T2 && !stop; c0 += 32) {
             const int c = c0 + lane;
-            int pw = 0;  // the last lane whose candidates start at or before c
-#pragma unroll
-            for (int st = 16; st; st >>= 1) {
-              const int pv = __shfl_sync(FULL, pre2, pw + st);
-              if (pv <= c) pw += st;
-            }
+            const unsigned s2 = __reduce_or_sync(FULL, cnt > 0 && (unsigned)(pre2 - c0) < 32u ? 1u << (pre2 - c0) : 0u);
+            const int pw = own2[before2 + __popc(s2 & upto)];  // the lane whose candidate c is
+            before2 += __popc(s2);
             const int pi0 = __shfl_sync(FULL, i0, pw), pi1 = __shfl_sync(FULL, oi1, pw);
             const int plo = __shfl_sync(FULL, lo, pw), ppre = __shfl_sync(FULL, pre2, pw);
             const float ptl = __shfl_sync(FULL, tl01, pw);
