@@ -188,9 +188,10 @@ int m3e_select_frames_debug(m3e_ctx* ctx, int form, const int32_t* d_hits, const
  * enqueueing; the results are in h_keep/h_reason once `stream` has reached the
  * call (the caller's stream waits for both internal streams).  Host buffers that
  * are page-locked copy at full speed; others work, more slowly.  Consecutive calls
- * on one context must be ordered by the caller's stream. */
+ * on one context must be ordered by the caller's stream.  A batch of at most 8192
+ * frames is copied and selected in order on `stream` itself. */
 /* Settings of m3e_select_frames_host: at most max_chunks chunks (1..64, default
- * 16; a chunk holds at least 50,000 frames unless the batch is smaller), a wait of
+ * 16; a chunk holds at least 12,500 frames unless the batch is smaller), a wait of
  * at most wait_ms (1..60,000, default 2,000) for one chunk, and drop_chunk: -1 in
  * normal use; k >= 0 leaves chunk k's flag unset, so that stage 1 runs out of its
  * wait (a test of the bounded wait; the call then latches M3E_ETIMEOUT). */
