@@ -272,10 +272,11 @@ int grow(T*& ptr, int64_t& cap, int64_t need, size_t elem, const char* what) {
 // those of the throughput mix (85 hits, 44 triplets) with a margin; a batch of denser
 // frames needs more, so up to the scratch of ROOMY_FRAMES frames a batch gets the second,
 // roomier figure (20,001 frames of 32 tracks, 137 hits and 108 triplets each: 7,000 frames
-// deferred and 855 us with the first figures alone).
+// deferred and 855 us with the first figures alone, 362 us with these; more costs a
+// millisecond of allocation per GB when a context is prepared).
 constexpr int64_t ROOMY_FRAMES = 1 << 20;
-constexpr int64_t HITS_PER_FRAME[2] = {128, 512};
-constexpr int64_t TRIPLETS_PER_FRAME[2] = {64, 512};
+constexpr int64_t HITS_PER_FRAME[2] = {128, 384};
+constexpr int64_t TRIPLETS_PER_FRAME[2] = {64, 256};
 constexpr int64_t COMBOS_PER_FRAME[2] = {192, 384};
 
 int64_t scratch_entries(const int64_t (&per_frame)[2], int64_t nf) {
