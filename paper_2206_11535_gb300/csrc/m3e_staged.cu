@@ -275,6 +275,14 @@ __global__ void __launch_bounds__(128, 8)  // 8 CTAs per SM (64 registers: the f
   }
 }
 
+__device__ __forceinline__ void load_circle(const float4* __restrict__ rec, int64_t k, float& cx, float& cy,
+                                            float& rt) {
+  const float4 a = __ldg(rec + 4 * k);
+  cx = a.x;
+  cy = a.y;
+  rt = a.z;
+}
+
 // ---- stage 3: warp per frame, track cap and energy test (NOST: the instance for
 // runs without statistics).
 // A warp takes P.grab frames at a time: their states are read together, a lane each, the
@@ -284,12 +292,16 @@ __global__ void __launch_bounds__(128, 8)  // 8 CTAs per SM (64 registers: the f
 // SM at 48 registers; 12 spill and take 15% longer): 1e6 throughput frames 854 -> 719 us,
 // 200,000 uneven frames 541 -> 283 us, most of that from frames that stop at the combination
 // cap.  Taking 16 frames at a time cost 745 and 535 us (heavy frames queue in one warp).
+// Before they are written the combinations go through the vertex's first two steps, which
+// three in four do not survive: their gathers of track circles from DRAM bounded stage 4 and
+// fit beside the arithmetic here (this stage 719 -> 817 us, stage 4 399 -> 225 us).
 template <bool DEBUG, bool NOST = false>
 __global__ void __launch_bounds__(S3_WARPS * 32, 10)
     k_stage3(const __grid_constant__ DevCfg C, const __grid_constant__ KParams P, const __grid_constant__ SParams S) {
   __shared__ S3Sm<!NOST> smem[S3_WARPS];
   S3Sm<!NOST>& sm = smem[threadIdx.x >> 5];
   const int lane = threadIdx.x & 31;
+  const unsigned below = (1u << lane) - 1u;
   if (!NOST)
     for (int k = lane; k < ST_REASON0 + 8; k += 32) sm.acc[k] = 0;
   __syncwarp();
@@ -347,7 +359,31 @@ __global__ void __launch_bounds__(S3_WARPS * 32, 10)
     auto flush = [&]() {
       if (fill == 0) return;
       __syncwarp();
-      const long long cb = allocate(fill);
+      if (!DEBUG) {
+        // only the combinations that the vertex's first two steps leave go on; the others
+        // decide nothing (the candidate record wants them all)
+        int kept = 0;
+        for (int t0 = 0; t0 < fill; t0 += 32) {
+          const int t = t0 + lane;
+          bool keep = t < fill;
+          int4 q = make_int4(0, 0, 0, 0);
+          if (keep) {
+            q = sm.buf[t];
+            float c[9];
+            load_circle(S.trec, q.y, c[0], c[1], c[2]);
+            load_circle(S.trec, q.z, c[3], c[4], c[5]);
+            load_circle(S.trec, q.w, c[6], c[7], c[8]);
+            keep = vertex_prefilter(c, c + 3, c + 6, C.isect_lim) == 2;
+          }
+          const unsigned m = __ballot_sync(FULL, keep);
+          __syncwarp();
+          if (keep) sm.buf[kept + __popc(m & below)] = q;  // never beyond the entries read
+          kept += __popc(m);
+          __syncwarp();
+        }
+        fill = kept;
+      }
+      const long long cb = fill ? allocate(fill) : 0;
       for (int t = lane; cb >= 0 && t < fill; t += 32) S.combo[cb + t] = sm.buf[t];
       placed(cb);
       fill = 0;
@@ -442,16 +478,9 @@ __global__ void __launch_bounds__(S3_WARPS * 32, 10)
 // does not intersect, or no intersection inside the target filter).  Each warp
 // therefore runs those steps on 32 combinations at a time, appends the survivors
 // to a queue in shared memory, and runs the full vertex on 32 queued survivors at
-// a time, so that all lanes do the expensive part together.
+// a time, so that all lanes do the expensive part together.  In a decision-only run stage 3
+// has already dropped the others, except in frames with more combinations than its buffer.
 constexpr int S4_WARPS = 4;
-
-__device__ __forceinline__ void load_circle(const float4* __restrict__ rec, int64_t k, float& cx, float& cy,
-                                            float& rt) {
-  const float4 a = __ldg(rec + 4 * k);
-  cx = a.x;
-  cy = a.y;
-  rt = a.z;
-}
 
 template <bool DEBUG>
 __device__ __forceinline__ void stage4_dump(const DevCfg& C, const KParams& P, const SParams& S, int64_t i,
