@@ -327,7 +327,7 @@ int ensure_scratch(Scratch& sc, int64_t nf, bool staged) {
     int64_t c0 = sc.trip_cap, c1 = sc.trip_cap, c2 = sc.trip_cap;
     rc = grow(sc.trip, c0, tc, sizeof(int4), "triplets");
     if (!rc) rc = grow(sc.tek, c1, tc, sizeof(float2), "track energies");
-    if (!rc) rc = grow(sc.trec, c2, tc, 4 * sizeof(float4), "track records");
+    if (!rc) rc = grow(sc.trec, c2, tc, 2 * sizeof(float4), "track records");
     if (rc) return rc;
     sc.trip_cap = tc;
   }

@@ -662,8 +662,7 @@ __device__ __forceinline__ void track_record(const float4& p0, const float4& p1,
   tr[13] = eps;
 }
 
-// Track record layout (16 floats, also the global record of the staged form):
-// cx cy rt R ct st p E sms h0x h0y h0z ah0 eps - -
+// Track record layout (14 floats): cx cy rt R ct st p E sms h0x h0y h0z ah0 eps
 template <int CK>
 __device__ __forceinline__ void store_track(TrkSoA<CK>& T, int k, const float* tr, int tid) {
   T.cx[k] = tr[0];
@@ -698,14 +697,28 @@ __device__ __forceinline__ TrackR load_track(const TrkSoA<CK>& T, int k) {
   return t;
 }
 
-__device__ __forceinline__ TrackR load_track(const float4* __restrict__ rec, int64_t k) {
-  const float4 a = __ldg(rec + 4 * k), b = __ldg(rec + 4 * k + 1), c = __ldg(rec + 4 * k + 2),
-               d = __ldg(rec + 4 * k + 3);
+// The global record of the staged form, one 32-byte sector: cx cy rt R, ct st ah0 and the
+// layer-0 hit's place among the sorted hits, complemented for a negative charge.  Momentum
+// and scattering width follow from R by the operations of track_record (E is not filled).
+// With 64 bytes the track stage of 1e6 throughput frames took 2334 us instead of 2317, and
+// the scratch a third more.
+__device__ __forceinline__ void store_record(float4* rec, int64_t k, const float* tr, int hit) {
+  rec[2 * k] = make_float4(tr[0], tr[1], tr[2], tr[3]);
+  rec[2 * k + 1] = make_float4(tr[4], tr[5], tr[12], __int_as_float(tr[13] > 0.f ? hit : ~hit));
+}
+__device__ __forceinline__ TrackR load_track(const float4* __restrict__ rec, const float4* __restrict__ hits, int64_t k,
+                                             const DevCfg& C) {
+  const float4 a = __ldg(rec + 2 * k), b = __ldg(rec + 2 * k + 1);
+  const int h = __float_as_int(b.w);
+  const float4 q = __ldg(hits + (h < 0 ? ~h : h));
   TrackR t;
   t.cx = a.x; t.cy = a.y; t.rt = a.z; t.R = a.w;
-  t.ct = b.x; t.st = b.y; t.p = b.z; t.E = b.w;
-  t.sms = c.x; t.h0x = c.y; t.h0y = c.z; t.h0z = c.w;
-  t.ah0 = d.x; t.eps = d.y;
+  t.ct = b.x; t.st = b.y; t.ah0 = b.z;
+  t.p = __fmul_rn(C.kB, t.R);
+  t.E = 0.f;
+  t.sms = C.hl[0] / t.p;
+  t.h0x = q.x; t.h0y = q.y; t.h0z = q.z;
+  t.eps = h < 0 ? -1.f : 1.f;
   return t;
 }
 

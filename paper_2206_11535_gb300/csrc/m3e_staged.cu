@@ -250,11 +250,7 @@ __global__ void __launch_bounds__(128, 8)  // 8 CTAs per SM (64 registers: the f
       float tk[14];
       track_record(v.pos(i0), v.pos(i1), o, C, tk);
       te = make_float2(tk[13] * tk[7], pz_track(tk[6], tk[4]));  // what the energy test reads
-      float4* q = S.trec + 4 * i;
-      q[0] = make_float4(tk[0], tk[1], tk[2], tk[3]);
-      q[1] = make_float4(tk[4], tk[5], tk[6], tk[7]);
-      q[2] = make_float4(tk[8], tk[9], tk[10], tk[11]);
-      q[3] = make_float4(tk[12], tk[13], 0.f, 0.f);
+      store_record(S.trec, i, tk, r.y + i0);
     }
     S.tek[i] = te;
     if (DEBUG) {
@@ -277,7 +273,7 @@ __global__ void __launch_bounds__(128, 8)  // 8 CTAs per SM (64 registers: the f
 
 __device__ __forceinline__ void load_circle(const float4* __restrict__ rec, int64_t k, float& cx, float& cy,
                                             float& rt) {
-  const float4 a = __ldg(rec + 4 * k);
+  const float4 a = __ldg(rec + 2 * k);
   cx = a.x;
   cy = a.y;
   rt = a.z;
@@ -486,7 +482,7 @@ template <bool DEBUG>
 __device__ __forceinline__ void stage4_dump(const DevCfg& C, const KParams& P, const SParams& S, int64_t i,
                                             const int4& r, const VtxOut& v, const TrackR& A, const TrackR& B,
                                             const TrackR& E) {
-  const float esum = A.E + B.E + E.E;
+  const float esum = fabsf(S.tek[r.y].x) + fabsf(S.tek[r.z].x) + fabsf(S.tek[r.w].x);
   const int f = r.x;
   const int c = (int)(i - S.fcbase[f]);
   if (c < P.dump.cap_combo) {
@@ -544,7 +540,7 @@ __global__ void __launch_bounds__(S4_WARPS * 32, 8)  // 8 CTAs per SM (64 regist
           const int st = vertex_prefilter(ca, cb, ce, C.isect_lim);
           cand = st == 2;
           if (DEBUG && !cand) {  // record the combination with its early status (the same geometry)
-            const TrackR A = load_track(S.trec, r.y), B = load_track(S.trec, r.z), E = load_track(S.trec, r.w);
+            const TrackR A = load_track(S.trec, S.hp, r.y, C), B = load_track(S.trec, S.hp, r.z, C), E = load_track(S.trec, S.hp, r.w, C);
             stage4_dump<DEBUG>(C, P, S, i, r, vertex(A, B, E, C), A, B, E);
           }
         }
@@ -559,7 +555,7 @@ __global__ void __launch_bounds__(S4_WARPS * 32, 8)  // 8 CTAs per SM (64 regist
       if (lane < take) {
         const int64_t i = q[qn - take + lane];
         const int4 r = S.combo[i];
-        const TrackR A = load_track(S.trec, r.y), B = load_track(S.trec, r.z), E = load_track(S.trec, r.w);
+        const TrackR A = load_track(S.trec, S.hp, r.y, C), B = load_track(S.trec, S.hp, r.z, C), E = load_track(S.trec, S.hp, r.w, C);
         const VtxOut v = vertex(A, B, E, C);
         nv += v.status == 2;
         if (!NOST && P.stats && v.status == 2)
