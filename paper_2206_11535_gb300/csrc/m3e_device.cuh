@@ -1139,7 +1139,7 @@ __device__ __forceinline__ uint32_t phi_mask(const float* xs, const float* ys, i
                                              unsigned long long yy, float c) {
   const unsigned long long mc = pack2(-c, -c);
   uint32_t m = 0u;
-#pragma unroll 2
+#pragma unroll 1
   for (int q = ((n + 3) & ~3) - 4; q >= 0; q -= 4) {
     const ulonglong2 X = *reinterpret_cast<const ulonglong2*>(xs + q);
     const ulonglong2 Y = *reinterpret_cast<const ulonglong2*>(ys + q);
@@ -1277,11 +1277,14 @@ __device__ __forceinline__ void warp_cuts(S& sm, const DevCfg& C, bool stats, un
     }
     if (pc) {
       int wpos = pre;
+#pragma unroll 1
       for (uint32_t m = a0; m; m &= m - 1u) sm.p01[wpos++] = (uint16_t)((__ffs(m) - 1) | (lane << 8));
+#pragma unroll 1
       for (uint32_t m = a1; m; m &= m - 1u) sm.p01[wpos++] = (uint16_t)((__ffs(m) + 31) | (lane << 8));
     }
     __syncwarp();
     // 3. the pairs, 32 at a time
+#pragma unroll 1
     for (int k0 = 0; k0 < T; k0 += 32) {
       const int k = k0 + lane;
       const int pair = k < T ? sm.p01[k] : 0;
@@ -1312,18 +1315,16 @@ __device__ __forceinline__ void warp_cuts(S& sm, const DevCfg& C, bool stats, un
       for (int c0 = 0; c0 < ctot; c0 += W_CAND) {
         // each lane lists its candidates numbered c0 .. c0 + W_CAND - 1: pair lane, z-order position
         int idx = cpre - c0;
-        if (ctot <= W_CAND) {  // all of them fit: the usual case
-          for (uint32_t m = cl; m; m &= m - 1u) sm.cand[idx++] = (uint16_t)((lane << 6) | (__ffs(m) - 1));
-          for (uint32_t m = ch; m; m &= m - 1u) sm.cand[idx++] = (uint16_t)((lane << 6) | (__ffs(m) + 31));
-        } else {
-          for (uint32_t m = cl; m; m &= m - 1u, ++idx)
-            if (idx >= 0 && idx < W_CAND) sm.cand[idx] = (uint16_t)((lane << 6) | (__ffs(m) - 1));
-          for (uint32_t m = ch; m; m &= m - 1u, ++idx)
-            if (idx >= 0 && idx < W_CAND) sm.cand[idx] = (uint16_t)((lane << 6) | (__ffs(m) + 31));
-        }
+#pragma unroll 1
+        for (uint32_t m = cl; m; m &= m - 1u, ++idx)
+          if ((unsigned)idx < (unsigned)W_CAND) sm.cand[idx] = (uint16_t)((lane << 6) | (__ffs(m) - 1));
+#pragma unroll 1
+        for (uint32_t m = ch; m; m &= m - 1u, ++idx)
+          if ((unsigned)idx < (unsigned)W_CAND) sm.cand[idx] = (uint16_t)((lane << 6) | (__ffs(m) + 31));
         __syncwarp();
         // 4. the exact tests, 32 candidates at a time
         const int ne = min(ctot - c0, W_CAND);
+#pragma unroll 1
         for (int e0 = 0; e0 < ne; e0 += 32) {
           const int e = e0 + lane;
           const int ent = e < ne ? sm.cand[e] : 0;

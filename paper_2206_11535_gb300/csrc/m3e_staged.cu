@@ -54,6 +54,7 @@ __device__ __forceinline__ bool emit_frame(const G& g, Sm& sm, const DevCfg& C, 
   const long long hb = P.off[f] - P.off_base;
   const bool hits_fit = hb + n <= S.hits_cap;
   const int l3s = sm.bstart[3 * NB];  // phi of a sorted hit serves only the layer-3 search of stage 2
+#pragma unroll 1
   for (int i = g.rank(); hits_fit && i < n; i += G::N) {
     const float2 p = sm.xy[i];
     S.hp[hb + i] = make_float4(p.x, p.y, sm.z[i], i >= l3s ? sm.phi[i] : 0.f);
@@ -75,7 +76,9 @@ __device__ __forceinline__ bool emit_frame(const G& g, Sm& sm, const DevCfg& C, 
     for (int64_t t = tb + g.rank(); t < S.trip_cap && t < tb + ntrip; t += G::N) S.trip[t] = make_int4(-1, 0, 0, 0);
     return false;
   }
+#pragma unroll 1
   for (int b = g.rank(); b < NL3; b += G::N) S.l3[(int64_t)f * NL3 + b] = sm.bstart[3 * NB + b];
+#pragma unroll 1
   for (int t = g.rank(); t < ntrip; t += G::N) {
     const auto q = sm.u.trip[t];
     S.trip[tb + t] = make_int4(f, (int)hb, (int)q.x | ((int)q.y << 16), (int)q.z);
@@ -159,8 +162,10 @@ __device__ bool gate_wait(const KParams& P, int k) {
 // Bound by instruction issue and shared-memory latency (1,956 warp instructions per
 // throughput frame at 68% issue active; l1tex 65% busy, most of it the table gathers): 1e6
 // throughput frames 2.36 -> 2.15 ms with the packed partner masks, one decode per hit and no
-// address list, at 64 registers and 8 CTAs per SM (2.20 ms at 56 registers and 9 CTAs), and
-// 2.09 ms with x and y in one copy per hit.
+// address list, at 64 registers and 8 CTAs per SM (2.20 ms at 56 registers and 9 CTAs),
+// 2.09 ms with x and y in one copy per hit, and 2.02 ms with its loops rolled: a warp is
+// seldom where another one is, so every instruction fetched less counts (the masks unrolled
+// by 4 instead of 1: 2.27 ms).
 template <bool DEBUG, bool GATED = false, bool NOST = false>
 __global__ void __launch_bounds__(WARPS_PER_CTA * 32)
     k_stage1(const __grid_constant__ DevCfg C, const __grid_constant__ KParams P, const __grid_constant__ SParams S) {
