@@ -316,7 +316,7 @@ int ensure_scratch(Scratch& sc, int64_t nf, bool staged) {
   }
   if (nf > sc.frames_cap) {
     int64_t c0 = sc.frames_cap, c1 = sc.frames_cap, c2 = sc.frames_cap;
-    rc = grow(sc.l3, c0, nf, (NB + 1) * sizeof(uint16_t), "layer-3 bins");
+    rc = grow(sc.l3, c0, nf, (NB + 2) * sizeof(uint16_t), "layer-3 bins");
     if (!rc) rc = grow(sc.fint, c1, nf, 4 * sizeof(int), "frame state");
     if (!rc) rc = grow(sc.fcbase, c2, nf, sizeof(long long), "frame combination bases");
     if (rc) return rc;

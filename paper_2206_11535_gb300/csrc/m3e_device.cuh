@@ -63,7 +63,7 @@ struct FrameSm {
   alignas(16) float2 xy[CH];
   float z[CH], phi[CH];         // phi: layer-3 hits only (the 4th-hit search)
   uint16_t inidx[IDX ? CH : 1];
-  uint16_t bstart[NBK + 1];
+  uint16_t bstart[NBK + 2];       // one more than needed: read in pairs
   uint32_t bcur[kPackB ? NBK / 4 : NBK];  // bucket counts, then cursors
   // warp stage, selection cuts (warp_cuts): x and y of the layer-0 hits apart, the layer-2
   // hits in z-bin order (bin starts zbs; z and sorted index in zzi), the (layer-1 hit, Phi01 partner) pairs of a

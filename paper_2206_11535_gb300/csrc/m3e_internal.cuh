@@ -107,7 +107,7 @@ struct SParams {
   int* list1b;                 // frames deferred by the middle tier of stage 1
   int* list2;                  // frames deferred by the top tier of stage 1 and by stage 3
   int* lcount;                 // [0] list1 count, [1] list2 count, [2] list1b count
-  uint16_t* l3;                // [F][NB + 1] layer-3 phi-bin starts, frame-relative
+  uint16_t* l3;                // [F][NB + 2] layer-3 phi-bin starts, frame-relative (the last unused)
   int *fstate, *ftbase, *fntrip, *ffound;  // per frame: state, triplet range, vertex found
   long long* fcbase;           // per frame: first combination (candidate record only)
   int4* trip;                  // {frame, first sorted hit, i0 | i1 << 16, i2} (frame-relative indices), frame -1 = unused
