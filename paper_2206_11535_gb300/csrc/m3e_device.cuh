@@ -396,6 +396,8 @@ struct SmHits {
   const S& s;
   __device__ __forceinline__ float4 pos(int i) const { const float2 p = s.xy[i]; return make_float4(p.x, p.y, s.z[i], s.phi[i]); }
   __device__ __forceinline__ int l3(int b) const { return s.bstart[3 * NB + b]; }  // layer-3 bin starts
+  __device__ __forceinline__ int l3_first() const { return l3(0); }
+  __device__ __forceinline__ int l3_end() const { return l3(NB); }
 };
 
 // The first triplet fit's values that the global fit and the track record need,
@@ -440,13 +442,17 @@ __device__ __forceinline__ TFitF unpark_fit(const FitPark& pk) {
   return f;
 }
 
+template <bool EARLY>                // EARLY: the layer-3 range is loaded with the triplet's hits
 struct GHits {                       // one 16-byte load per hit
   static constexpr bool kPark = true;
   const float4* __restrict__ ps;
   const uint16_t* __restrict__ l3s;  // NB + 1 layer-3 bin starts, frame-relative
   FitPark* park;
+  unsigned range;                    // EARLY: layer-3 hits, first | end << 16
   __device__ __forceinline__ float4 pos(int i) const { return __ldg(ps + i); }
   __device__ __forceinline__ int l3(int b) const { return __ldg(l3s + b); }
+  __device__ __forceinline__ int l3_first() const { return EARLY ? (int)(range & 0xffff) : l3(0); }
+  __device__ __forceinline__ int l3_end() const { return EARLY ? (int)(range >> 16) : l3(NB); }
 };
 
 // ------------------------------------------------------------------ track reconstruction
@@ -569,7 +575,7 @@ __device__ __forceinline__ TrackOut build_track(const V& v, const DevCfg& C, int
       mb = mm;
     }
   };
-  const int l3a = v.l3(0), l3e = v.l3(NB);
+  const int l3a = v.l3_first(), l3e = v.l3_end();
   if (l3e - l3a <= SCAN3_MAX) {
     // few layer-3 hits: a straight scan, whose loads do not depend on each other.
     // It reads no addresses: it notes whether another hit has the same metric as
@@ -579,7 +585,7 @@ __device__ __forceinline__ TrackOut build_track(const V& v, const DevCfg& C, int
       best = l3a;
       mb = metric(v.pos(l3a));
     }
-#pragma unroll 4
+#pragma unroll 6
     for (int j = l3a + 1; j < l3e; ++j) {
       const float mm = metric(v.pos(j));
       if (mm < mb) {
