@@ -113,7 +113,7 @@ struct SParams {
   int4* trip;                  // {frame, first sorted hit, i0 | i1 << 16, i2} (frame-relative indices), frame -1 = unused
   float2* tek;                 // per triplet: (eps E, P_z) of a kept track, (0, 0) otherwise
   float4* trec;                // per triplet: 32-byte track record when kept (store_record)
-  int4* combo;                 // {frame, triplet a, triplet b, triplet e-}, frame -1 = unused
+  int4* combo;                 // {frame, triplet a (FILTERED: sign bit), triplet b, triplet e-}, frame -1 = unused
   unsigned long long* counters;  // [0] triplets, [1] combinations, [2] stage-3 queue, [3] sorted hits
   int64_t trip_cap, combo_cap, hits_cap;
 };

@@ -19,6 +19,7 @@ namespace m3e {
 namespace {
 
 constexpr int NL3 = NB + 2;                        // layer-3 bin starts per frame (NB + 1, in whole words)
+constexpr int FILTERED = INT32_MIN;                // bit of a combination's first triplet: prefilter passed
 constexpr int S1_TRIP = 160;                       // stage-1 warp-tier triplet capacity
 // input indices only for the candidate record; the instance without statistics code has
 // no room for them
@@ -388,6 +389,7 @@ __global__ void __launch_bounds__(S3_WARPS * 32, 10)
           }
           const unsigned m = __ballot_sync(FULL, keep);
           __syncwarp();
+          q.y |= FILTERED;
           if (keep) sm.buf[kept + __popc(m & below)] = q;  // never beyond the entries read
           kept += __popc(m);
           __syncwarp();
@@ -490,7 +492,11 @@ __global__ void __launch_bounds__(S3_WARPS * 32, 10)
 // therefore runs those steps on 32 combinations at a time, appends the survivors
 // to a queue in shared memory, and runs the full vertex on 32 queued survivors at
 // a time, so that all lanes do the expensive part together.  In a decision-only run stage 3
-// has already dropped the others, except in frames with more combinations than its buffer.
+// has already dropped the others and marked these (FILTERED), except in frames with more
+// combinations than its buffer.
+// Bound by the latency of the track records and by spills: 1e6 throughput frames 229 us at 64
+// registers (8 CTAs per SM) with every combination filtered again, 217 without that, 213 at 80
+// registers, 191 at 96, 200 at 128 (no spills, 4 CTAs per SM); 200,000 uneven frames 68 -> 59.
 constexpr int S4_WARPS = 4;
 
 template <bool DEBUG>
@@ -523,7 +529,7 @@ __device__ __forceinline__ void stage4_dump(const DevCfg& C, const KParams& P, c
 }
 
 template <bool DEBUG, bool NOST = false>
-__global__ void __launch_bounds__(S4_WARPS * 32, 8)  // 8 CTAs per SM (64 registers)
+__global__ void __launch_bounds__(S4_WARPS * 32, 5)  // 96 registers
     k_stage4(const __grid_constant__ DevCfg C, const __grid_constant__ KParams P, const __grid_constant__ SParams S) {
   __shared__ long long queue[S4_WARPS][64];
   long long* q = queue[threadIdx.x >> 5];
@@ -535,23 +541,27 @@ __global__ void __launch_bounds__(S4_WARPS * 32, 8)  // 8 CTAs per SM (64 regist
   int qn = 0;
   unsigned nv = 0, nvo = 0;
   int64_t base = ((int64_t)blockIdx.x * S4_WARPS + (threadIdx.x >> 5)) * 32;
-  // the combination records are loaded one step ahead; the three circles are read
-  // together with the frame's state, before it is known whether they are needed
-  int4 rn = base + lane < n ? S.combo[base + lane] : make_int4(-1, 0, 0, 0);
+  // the combination records are fetched into L1 one step ahead; the three circles are
+  // read together with the frame's state, before it is known whether they are needed
   for (;; base += stride) {
     const bool more = base < n;  // uniform in the warp
     if (more) {
       const int64_t i = base + lane;
-      const int4 r = rn;
-      if (i + stride < n) rn = S.combo[i + stride];
+      const int4 r = i < n ? S.combo[i] : make_int4(-1, 0, 0, 0);
+      if (i + stride < n) asm volatile("prefetch.global.L1 [%0];" ::"l"(S.combo + i + stride));
       bool cand = false;
       if (i < n && r.x >= 0) {
         const int f = r.x;
         float ca[3], cb[3], ce[3];
-        load_circle(S.trec, r.y, ca[0], ca[1], ca[2]);
-        load_circle(S.trec, r.z, cb[0], cb[1], cb[2]);
-        load_circle(S.trec, r.w, ce[0], ce[1], ce[2]);
-        if (DEBUG || !*((volatile int*)S.ffound + f)) {
+        if (DEBUG || r.y >= 0) {
+          load_circle(S.trec, r.y, ca[0], ca[1], ca[2]);
+          load_circle(S.trec, r.z, cb[0], cb[1], cb[2]);
+          load_circle(S.trec, r.w, ce[0], ce[1], ce[2]);
+        }
+        const bool open = DEBUG || !*((volatile int*)S.ffound + f);
+        if (!DEBUG && r.y < 0) {
+          cand = open;
+        } else if (open) {
           const int st = vertex_prefilter(ca, cb, ce, C.isect_lim);
           cand = st == 2;
           if (DEBUG && !cand) {  // record the combination with its early status (the same geometry)
@@ -569,7 +579,8 @@ __global__ void __launch_bounds__(S4_WARPS * 32, 8)  // 8 CTAs per SM (64 regist
       const int take = qn < 32 ? qn : 32;
       if (lane < take) {
         const int64_t i = q[qn - take + lane];
-        const int4 r = S.combo[i];
+        int4 r = S.combo[i];
+        r.y &= ~FILTERED;
         const TrackR A = load_track(S.trec, S.hp, r.y, C), B = load_track(S.trec, S.hp, r.z, C), E = load_track(S.trec, S.hp, r.w, C);
         const VtxOut v = vertex(A, B, E, C);
         nv += v.status == 2;
