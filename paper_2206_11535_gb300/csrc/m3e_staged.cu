@@ -161,8 +161,8 @@ __device__ bool gate_wait(const KParams& P, int k) {
 // GATED (host entry point): the hits arrive while the kernel runs; a frame is
 // taken only after its chunk's arrival flag, and the hits are read past L1.
 // NOST: the instance for runs without statistics (no statistics code at all).
-// Bound by instruction issue and shared-memory latency (1,956 warp instructions per
-// throughput frame at 68% issue active; l1tex 65% busy, most of it the table gathers): 1e6
+// Bound by instruction issue and shared-memory latency (1,854 warp instructions per
+// throughput frame at 66% issue active; shared-memory loads are the largest stall): 1e6
 // throughput frames 2.36 -> 2.15 ms with the packed partner masks, one decode per hit and no
 // address list, at 64 registers and 8 CTAs per SM (2.20 ms at 56 registers and 9 CTAs),
 // 2.09 ms with x and y in one copy per hit, and 2.02 ms with its loops rolled: a warp is
@@ -231,7 +231,7 @@ __global__ void __launch_bounds__(NT)
 
 // ---- stage 2: one thread per selected triplet
 // Bound by issue and the latency of the hit loads (2,060 warp instructions per throughput frame
-// at 71% issue active, 27 of 32 lanes, 27 warps per SM).  What it holds across the fits counts
+// at 73% issue active, 27 of 32 lanes, 27 warps per SM).  What it holds across the fits counts
 // twice, as a spill and as a load issued late: with the next record fetched into L1 instead of
 // into four registers, 32-bit indices, the layer-3 range loaded beside the triplet's hits and
 // the layer-3 scan unrolled by 6, 1e6 throughput frames take 2.26 ms instead of 2.32, without
@@ -300,8 +300,8 @@ __device__ __forceinline__ void load_circle(const float4* __restrict__ rec, int6
 // A warp takes P.grab frames at a time: their states are read together, a lane each, the
 // tracks of the next frame are loaded while one is tested, and the combinations of all of
 // them are written behind one allocation, a fourth of the atomics on the one counter.
-// Bound by issue (770 warp instructions per throughput frame, 73% issue active, 10 CTAs per
-// SM at 48 registers; 12 spill and take 15% longer): 1e6 throughput frames 854 -> 719 us,
+// Bound by issue (861 warp instructions per throughput frame, 70% issue active, 10 CTAs per
+// SM at 48 registers; 9 CTAs at 56 take 2% longer, 12 CTAs 15%): 1e6 throughput frames 854 -> 719 us,
 // 200,000 uneven frames 541 -> 283 us, most of that from frames that stop at the combination
 // cap.  Taking 16 frames at a time cost 745 and 535 us (heavy frames queue in one warp).
 // Before they are written the combinations go through the vertex's first two steps, which
