@@ -298,7 +298,7 @@ __device__ __forceinline__ void load_circle(const float4* __restrict__ rec, int6
 // ---- stage 3: warp per frame, track cap and energy test (NOST: the instance for
 // runs without statistics).
 // A warp takes P.grab frames at a time: their states are read together, a lane each, the
-// tracks of the next frame are loaded while one is tested, and the combinations of all of
+// tracks of the next frame are fetched into L1 while one is tested, and the combinations of all of
 // them are written behind one allocation, a fourth of the atomics on the one counter.
 // Bound by issue (861 warp instructions per throughput frame, 70% issue active, 10 CTAs per
 // SM at 48 registers; 9 CTAs at 56 take 2% longer, 12 CTAs 15%): 1e6 throughput frames 854 -> 719 us,
@@ -306,7 +306,9 @@ __device__ __forceinline__ void load_circle(const float4* __restrict__ rec, int6
 // cap.  Taking 16 frames at a time cost 745 and 535 us (heavy frames queue in one warp).
 // Before they are written the combinations go through the vertex's first two steps, which
 // three in four do not survive: their gathers of track circles from DRAM bounded stage 4 and
-// fit beside the arithmetic here (this stage 719 -> 817 us, stage 4 399 -> 225 us).
+// fit beside the arithmetic here (this stage 719 -> 817 us, stage 4 399 -> 225 us).  The next
+// frame's tracks went into four registers at first, and the kernel spilled 148 bytes a thread;
+// fetched into L1 instead, 44 bytes and 793 us.
 template <bool DEBUG, bool NOST = false>
 __global__ void __launch_bounds__(S3_WARPS * 32, 10)
     k_stage3(const __grid_constant__ DevCfg C, const __grid_constant__ KParams P, const __grid_constant__ SParams S) {
@@ -402,19 +404,14 @@ __global__ void __launch_bounds__(S3_WARPS * 32, 10)
       fill = 0;
       __syncwarp();
     };
-    float2 n0 = make_float2(0.f, 0.f), n1 = n0;
-    if (todo) {
-      n0 = load(__ffs(todo) - 1, 0);
-      n1 = load(__ffs(todo) - 1, 32);
-    }
     while (todo) {
       const int j = __ffs(todo) - 1;
       todo &= todo - 1u;
       const int tb = __shfl_sync(FULL, tbase, j), nt = __shfl_sync(FULL, ntrip, j), fj = f0 + j;
-      const float2 te0 = n0, te1 = n1;
+      const float2 te0 = load(j, 0), te1 = load(j, 32);
       if (todo) {
-        n0 = load(__ffs(todo) - 1, 0);
-        n1 = load(__ffs(todo) - 1, 32);
+        const int tn = __shfl_sync(FULL, tbase, __ffs(todo) - 1), nn = __shfl_sync(FULL, ntrip, __ffs(todo) - 1);
+        if (4 * lane < nn && lane < 16) asm volatile("prefetch.global.L1 [%0];" ::"l"(S.tek + tn + 4 * lane));
       }
       // kept tracks of the frame's triplets, split by charge
       int npos = 0, nneg = 0;
