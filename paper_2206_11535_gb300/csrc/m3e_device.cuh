@@ -1258,14 +1258,14 @@ __device__ __forceinline__ void warp_cuts(S& sm, const DevCfg& C, bool stats, un
                  (s2 + nb2 > NB ? sm.bstart[2 * NB + s2 + nb2 - NB] - sm.bstart[2 * NB] : 0);
       }
     }
-    // 1. Phi01 and Phi12 partners as bit masks (lanes without a layer-1 hit test
-    // (0, 0), which passes neither cut)
+    // 1. Phi01 and Phi12 partners as bit masks (a lane without a layer-1 hit has none: its
+    // (0, 0) would pass a cut above pi/2)
     const unsigned long long xx = pack2(x1, x1), yy = pack2(y1, y1);
     const uint32_t a0 = phi_mask(sm.ox, sm.oy, min(n0, 32), xx, yy, C.c01);
     const uint32_t a1 = n0 > 32 ? phi_mask(sm.ox + 32, sm.oy + 32, n0 - 32, xx, yy, C.c01) : 0u;
     const uint32_t b0 = phi_mask(sm.zx, sm.zy, min(n2, 32), xx, yy, C.c12);
     const uint32_t b1 = n2 > 32 ? phi_mask(sm.zx + 32, sm.zy + 32, n2 - 32, xx, yy, C.c12) : 0u;
-    const int c01 = __popc(a0) + __popc(a1), c12all = __popc(b0) + __popc(b1);
+    const int c01 = has ? __popc(a0) + __popc(a1) : 0, c12all = __popc(b0) + __popc(b1);
     ntt += (unsigned)(c01 * c12all);
     // 2. the pairs whose layer-1 hit has Phi12 partners, listed by their layer-0 hit
     const int pc = c12all ? c01 : 0;
