@@ -37,7 +37,7 @@ def _stale(target: str, deps: list[str]) -> bool:
 def build(force: bool = False, verbose: bool = False, src_dir: str = SRC, out: str = OUT) -> str:
     """Compile the units of ``src_dir`` and link ``out`` (defaults: this package)."""
     hdrs = [os.path.join(src_dir, "m3e_internal.cuh"), os.path.join(src_dir, "m3e_device.cuh"),
-            os.path.join(ROOT, "include", "m3e.h"), __file__]
+            os.path.join(src_dir, "m3e_scratch.h"), os.path.join(ROOT, "include", "m3e.h"), __file__]
     objs = []
     jobs = []
     for u in UNITS:

@@ -10,6 +10,7 @@
 #include <vector>
 
 #include "m3e_internal.cuh"
+#include "m3e_scratch.h"
 
 using namespace m3e;
 
@@ -61,31 +62,6 @@ int m3e::m3e_set_error(int code, const char* fmt, ...) {
   va_end(ap);
   return code;
 }
-
-// Device scratch of one launch sequence: work queue, deferred-frame list and the
-// global candidate arrays of the staged form.  The context holds one set for the
-// device entry points and two for the double-buffered host entry point.
-struct Scratch {
-  int* work = nullptr;                      // [0] work-queue head, [1] list-1 count, [2] list-2 count
-  unsigned long long* counters = nullptr;   // staged: [0] triplets, [1] combinations, [2] stage-3 queue, [3] hits
-  int* defer = nullptr;                     // list 1: deferred frames
-  int* defer2 = nullptr;                    // list 2 (staged form)
-  int* defer1b = nullptr;                   // list 1b (staged form)
-  int64_t defer_cap = 0;
-  float* hf = nullptr;                      // hx, hy, hz, hphi
-  uint16_t* hidx = nullptr;
-  int64_t hits_cap = 0;
-  uint16_t* l3 = nullptr;
-  int* fint = nullptr;                      // fstate, ftbase, fntrip, ffound
-  long long* fcbase = nullptr;              // per frame: first combination
-  int64_t frames_cap = 0;
-  int4* trip = nullptr;
-  float2* tek = nullptr;
-  float4* trec = nullptr;
-  int64_t trip_cap = 0;
-  int4* combo = nullptr;
-  int64_t combo_cap = 0;
-};
 
 struct m3e_ctx {
   int device = 0;
@@ -255,103 +231,21 @@ KParams base_params(m3e_ctx* x, Scratch& sc) {
   return p;
 }
 
-template <class T>
-int grow(T*& ptr, int64_t& cap, int64_t need, size_t elem, const char* what) {
-  if (need <= cap) return M3E_OK;
-  if (ptr) CUDA_TRY(cudaFree(ptr));
-  ptr = nullptr;
-  cap = 0;
-  if (cudaMalloc(&ptr, elem * (size_t)need) != cudaSuccess) return fail(M3E_ENOMEM, "%s: %lld entries", what, (long long)need);
-  cap = need;
+// A failed allocation is reported by the call that made it and by no later one: the runtime's
+// last error would fail the next launch's check.
+int device_get(void** p, size_t bytes) {
+  if (cudaMalloc(p, bytes) == cudaSuccess) return M3E_OK;
+  cudaGetLastError();
+  *p = nullptr;
+  return fail(M3E_ENOMEM, "device memory: %zu bytes", bytes);
+}
+int device_put(void* p) {
+  if (p) CUDA_TRY(cudaFree(p));
   return M3E_OK;
 }
+constexpr ScratchMemory DEVICE_MEMORY = {device_get, device_put};
 
-// Scratch for a batch of nf frames (staged arrays only when staged).  The sorted hits,
-// triplets and combinations of a batch share its scratch, and frames that find it full go
-// to the CTA-per-frame kernel, which runs them many times slower.  The sizes per frame are
-// those of the throughput mix (85 hits, 44 triplets) with a margin; a batch of denser
-// frames needs more, so up to the scratch of ROOMY_FRAMES frames a batch gets the second,
-// roomier figure (20,001 frames of 32 tracks, 137 hits and 108 triplets each: 7,000 frames
-// deferred and 855 us with the first figures alone, 362 us with these; more costs a
-// millisecond of allocation per GB when a context is prepared).
-constexpr int64_t ROOMY_FRAMES = 1 << 20;
-constexpr int64_t HITS_PER_FRAME[2] = {128, 384};
-constexpr int64_t TRIPLETS_PER_FRAME[2] = {64, 256};
-constexpr int64_t COMBOS_PER_FRAME[2] = {192, 384};
-
-int64_t scratch_entries(const int64_t (&per_frame)[2], int64_t nf) {
-  // indices travel as int32 in the records: at most 2^31 - 2^16 entries
-  const int64_t lim = ((int64_t)1 << 31) - (1 << 16);
-  const int64_t roomy = std::min(per_frame[1] * nf, per_frame[0] * ROOMY_FRAMES);
-  return std::min(std::max({per_frame[0] * nf, roomy, (int64_t)1 << 16}), lim);
-}
-
-int ensure_scratch(Scratch& sc, int64_t nf, bool staged) {
-  const int64_t nh = scratch_entries(HITS_PER_FRAME, nf);
-  int64_t one = sc.work ? 1 : 0;
-  int rc = grow(sc.work, one, 1, 4 * sizeof(int), "work counters");
-  if (rc) return rc;
-  int64_t one2 = sc.counters ? 1 : 0;
-  rc = grow(sc.counters, one2, 1, 4 * sizeof(unsigned long long), "counters");
-  if (rc) return rc;
-  {
-    const int64_t dc = nf > 4096 ? nf : 4096;
-    if (dc > sc.defer_cap) {
-      int64_t c0 = sc.defer_cap, c1 = sc.defer_cap, c2 = sc.defer_cap;
-      rc = grow(sc.defer, c0, dc, sizeof(int), "deferred list");
-      if (!rc) rc = grow(sc.defer2, c1, dc, sizeof(int), "deferred list 2");
-      if (!rc) rc = grow(sc.defer1b, c2, dc, sizeof(int), "deferred list 1b");
-      if (rc) return rc;
-      sc.defer_cap = dc;
-    }
-  }
-  if (!staged) return M3E_OK;
-  int64_t hc = sc.hits_cap;
-  if (nh > hc) {
-    int64_t c0 = hc, c1 = hc;
-    rc = grow(sc.hf, c0, nh, 4 * sizeof(float), "sorted hits");
-    if (!rc) rc = grow(sc.hidx, c1, nh, sizeof(uint16_t), "sorted input indices");
-    if (rc) return rc;
-    sc.hits_cap = nh;
-  }
-  if (nf > sc.frames_cap) {
-    int64_t c0 = sc.frames_cap, c1 = sc.frames_cap, c2 = sc.frames_cap;
-    rc = grow(sc.l3, c0, nf, (NB + 2) * sizeof(uint16_t), "layer-3 bins");
-    if (!rc) rc = grow(sc.fint, c1, nf, 4 * sizeof(int), "frame state");
-    if (!rc) rc = grow(sc.fcbase, c2, nf, sizeof(long long), "frame combination bases");
-    if (rc) return rc;
-    sc.frames_cap = nf;
-  }
-  const int64_t tc = scratch_entries(TRIPLETS_PER_FRAME, nf);
-  if (tc > sc.trip_cap) {
-    int64_t c0 = sc.trip_cap, c1 = sc.trip_cap, c2 = sc.trip_cap;
-    rc = grow(sc.trip, c0, tc, sizeof(int4), "triplets");
-    if (!rc) rc = grow(sc.tek, c1, tc, sizeof(float2), "track energies");
-    if (!rc) rc = grow(sc.trec, c2, tc, 2 * sizeof(float4), "track records");
-    if (rc) return rc;
-    sc.trip_cap = tc;
-  }
-  const int64_t cc = scratch_entries(COMBOS_PER_FRAME, nf);
-  return grow(sc.combo, sc.combo_cap, cc, sizeof(int4), "combinations");
-}
-
-void free_scratch(Scratch& sc) {
-  cudaFree(sc.work);
-  cudaFree(sc.counters);
-  cudaFree(sc.defer);
-  cudaFree(sc.defer2);
-  cudaFree(sc.defer1b);
-  cudaFree(sc.hf);
-  cudaFree(sc.hidx);
-  cudaFree(sc.l3);
-  cudaFree(sc.fint);
-  cudaFree(sc.fcbase);
-  cudaFree(sc.trip);
-  cudaFree(sc.tek);
-  cudaFree(sc.trec);
-  cudaFree(sc.combo);
-  sc = Scratch();
-}
+int ensure_scratch(Scratch& sc, int64_t nf, bool staged) { return ensure_scratch(DEVICE_MEMORY, sc, nf, staged); }
 
 SParams staged_params(const Scratch& sc) {
   SParams s{};
@@ -540,9 +434,9 @@ int m3e_destroy(m3e_ctx* x) {
   cudaFree(x->row_lut);
   cudaFree(x->err);
   if (x->h_err) cudaFreeHost(x->h_err);
-  free_scratch(x->main);
+  free_scratch(DEVICE_MEMORY, x->main);
   for (int i = 0; i < 2; ++i) {
-    free_scratch(x->hsc[i]);
+    free_scratch(DEVICE_MEMORY, x->hsc[i]);
     cudaFree(x->d_hits[i]);
     cudaFree(x->d_off[i]);
     cudaFree(x->d_out[i]);
@@ -693,20 +587,10 @@ int m3e_select_frames_host(m3e_ctx* x, const int32_t* h_hits, const int64_t* h_o
   if (h_off[n] > h_off[0] && !h_hits) return fail(M3E_EINVAL, "hits is NULL");
   DeviceGuard guard(x->device);
   const int64_t total = h_off[n] - h_off[0];
-  rc = grow(x->d_hits[0], x->cap_hits[0], total + total / 4 + 1024, sizeof(int32_t), "staging hits");
+  rc = resize(DEVICE_MEMORY, x->cap_hits[0], total + total / 4 + 1024, {{x->d_hits[0], sizeof(int32_t)}});
+  if (!rc && n + 1 > x->cap_frames[0])
+    rc = resize(DEVICE_MEMORY, x->cap_frames[0], n + n / 4 + 1024, {{x->d_off[0], sizeof(int64_t)}, {x->d_out[0], 2}});
   if (rc) return rc;
-  if (n + 1 > x->cap_frames[0]) {
-    cudaFree(x->d_off[0]);
-    cudaFree(x->d_out[0]);
-    x->d_off[0] = nullptr;
-    x->d_out[0] = nullptr;
-    x->cap_frames[0] = 0;
-    const int64_t cap = n + n / 4 + 1024;
-    if (cudaMalloc(&x->d_off[0], sizeof(int64_t) * (cap + 1)) != cudaSuccess ||
-        cudaMalloc(&x->d_out[0], 2 * cap) != cudaSuccess)
-      return fail(M3E_ENOMEM, "staging frames");
-    x->cap_frames[0] = cap;
-  }
   const Route route = x->gate_drop < 0 ? route_of(FORM_STAGED, n, false, false, nullptr) : ROUTE_FORM;
   if (route != ROUTE_SMALL) rc = ensure_scratch(x->hsc[0], n, route == ROUTE_FORM);
   if (rc) return rc;
