@@ -209,7 +209,12 @@ int m3e_check(m3e_ctx* ctx, cudaStream_t stream);
 int m3e_set_launch(m3e_ctx* ctx, int frames_per_grab, int ctas_per_sm);
 
 /* Size the context's scratch for batches of up to max_frames frames, so that the
- * select calls that follow allocate nothing (required before m3e_graph_create). */
+ * select calls that follow allocate nothing (required before m3e_graph_create).
+ * About 27.5 KB of device memory per frame up to 260,000 frames (dense frames then
+ * stay in the throughput kernels), 9.5 GB at most up to 1,048,576 and 9.1 KB per
+ * frame beyond; where that much is not free, 9.1 KB per frame.  A select call on a
+ * batch larger than any before does the same by itself, m3e_select_frames_host once
+ * more for its own set. */
 int m3e_prepare(m3e_ctx* ctx, int64_t max_frames);
 
 /* One batch as a CUDA graph (the persistent batched form, captured once and

@@ -32,6 +32,7 @@ struct Scratch {
   int64_t trip_cap = 0;
   int4* combo = nullptr;
   int64_t combo_cap = 0;
+  int64_t lean_frames = 0;                  // batches up to this one have the first figures per frame only
 };
 
 // The memory calls: M3E_OK, or the code that the entry point returns (get: the array is null then).
@@ -77,18 +78,42 @@ inline int resize(const ScratchMemory& m, int64_t& cap, int64_t need, std::initi
 // those of the throughput mix (85 hits, 44 triplets) with a margin; a batch of denser
 // frames needs more, so up to the scratch of ROOMY_FRAMES frames a batch gets the second,
 // roomier figure (20,001 frames of 32 tracks, 137 hits and 108 triplets each: 7,000 frames
-// deferred and 855 us with the first figures alone, 362 us with these; more costs a
-// millisecond of allocation per GB when a context is prepared).
+// deferred and 855 us with the first figures alone, 348 us with these; more costs a
+// millisecond of allocation per GB when a context is prepared).  That is 27.5 KB a frame
+// instead of 9.1; where it does not fit, the first figures do, and only cost speed.
 constexpr int64_t ROOMY_FRAMES = 1 << 20;
 constexpr int64_t HITS_PER_FRAME[2] = {128, 384};
 constexpr int64_t TRIPLETS_PER_FRAME[2] = {64, 256};
 constexpr int64_t COMBOS_PER_FRAME[2] = {192, 384};
 
-inline int64_t scratch_entries(const int64_t (&per_frame)[2], int64_t nf) {
+inline int64_t scratch_entries(const int64_t (&per_frame)[2], int64_t nf, bool roomy) {
   // indices travel as int32 in the records: at most 2^31 - 2^16 entries
   const int64_t lim = ((int64_t)1 << 31) - (1 << 16);
-  const int64_t roomy = std::min(per_frame[1] * nf, per_frame[0] * ROOMY_FRAMES);
-  return std::min(std::max({per_frame[0] * nf, roomy, (int64_t)1 << 16}), lim);
+  const int64_t more = roomy ? std::min(per_frame[1] * nf, per_frame[0] * ROOMY_FRAMES) : 0;
+  return std::min(std::max({per_frame[0] * nf, more, (int64_t)1 << 16}), lim);
+}
+
+inline int resize_staged(const ScratchMemory& m, Scratch& sc, int64_t nf, bool roomy) {
+  int rc = resize(m, sc.hits_cap, scratch_entries(HITS_PER_FRAME, nf, roomy),
+                  {{sc.hf, 4 * sizeof(float)}, {sc.hidx, sizeof(uint16_t)}});
+  if (!rc)
+    rc = resize(m, sc.frames_cap, nf,
+                {{sc.l3, (NB + 2) * sizeof(uint16_t)}, {sc.fint, 4 * sizeof(int)}, {sc.fcbase, sizeof(long long)}});
+  if (!rc)
+    rc = resize(m, sc.trip_cap, scratch_entries(TRIPLETS_PER_FRAME, nf, roomy),
+                {{sc.trip, sizeof(int4)}, {sc.tek, sizeof(float2)}, {sc.trec, 2 * sizeof(float4)}});
+  if (!rc) rc = resize(m, sc.combo_cap, scratch_entries(COMBOS_PER_FRAME, nf, roomy), {{sc.combo, sizeof(int4)}});
+  return rc;
+}
+
+inline void free_staged(const ScratchMemory& m, Scratch& sc) {
+  for (const ScratchArray& a : {ScratchArray(sc.hf, 0), ScratchArray(sc.hidx, 0), ScratchArray(sc.l3, 0),
+                                ScratchArray(sc.fint, 0), ScratchArray(sc.fcbase, 0), ScratchArray(sc.trip, 0),
+                                ScratchArray(sc.tek, 0), ScratchArray(sc.trec, 0), ScratchArray(sc.combo, 0)}) {
+    m.put(*a.array);
+    *a.array = nullptr;
+  }
+  sc.hits_cap = sc.frames_cap = sc.trip_cap = sc.combo_cap = 0;
 }
 
 inline int ensure_scratch(const ScratchMemory& m, Scratch& sc, int64_t nf, bool staged) {
@@ -99,23 +124,21 @@ inline int ensure_scratch(const ScratchMemory& m, Scratch& sc, int64_t nf, bool 
     rc = resize(m, sc.defer_cap, std::max<int64_t>(nf, 4096),
                 {{sc.defer, sizeof(int)}, {sc.defer2, sizeof(int)}, {sc.defer1b, sizeof(int)}});
   if (rc || !staged) return rc;
-  rc = resize(m, sc.hits_cap, scratch_entries(HITS_PER_FRAME, nf),
-              {{sc.hf, 4 * sizeof(float)}, {sc.hidx, sizeof(uint16_t)}});
-  if (!rc)
-    rc = resize(m, sc.frames_cap, nf,
-                {{sc.l3, (NB + 2) * sizeof(uint16_t)}, {sc.fint, 4 * sizeof(int)}, {sc.fcbase, sizeof(long long)}});
-  if (!rc)
-    rc = resize(m, sc.trip_cap, scratch_entries(TRIPLETS_PER_FRAME, nf),
-                {{sc.trip, sizeof(int4)}, {sc.tek, sizeof(float2)}, {sc.trec, 2 * sizeof(float4)}});
-  if (!rc) rc = resize(m, sc.combo_cap, scratch_entries(COMBOS_PER_FRAME, nf), {{sc.combo, sizeof(int4)}});
+  // batches that are known not to fit with the roomy figures are not tried with them again:
+  // the arrays that serve them would be freed for it
+  const bool roomy = nf > sc.lean_frames;
+  rc = resize_staged(m, sc, nf, roomy);
+  if (rc == M3E_ENOMEM && roomy) {
+    free_staged(m, sc);
+    rc = resize_staged(m, sc, nf, false);
+    if (!rc) sc.lean_frames = nf;
+  }
   return rc;
 }
 
 inline void free_scratch(const ScratchMemory& m, Scratch& sc) {
-  for (void* a : {(void*)sc.work, (void*)sc.counters, (void*)sc.defer, (void*)sc.defer2, (void*)sc.defer1b, (void*)sc.hf,
-                  (void*)sc.hidx, (void*)sc.l3, (void*)sc.fint, (void*)sc.fcbase, (void*)sc.trip, (void*)sc.tek,
-                  (void*)sc.trec, (void*)sc.combo})
-    m.put(a);
+  free_staged(m, sc);
+  for (void* a : {(void*)sc.work, (void*)sc.counters, (void*)sc.defer, (void*)sc.defer2, (void*)sc.defer1b}) m.put(a);
   sc = Scratch();
 }
 

@@ -85,3 +85,31 @@ for (int k = 0; k < 40; ++k) {
   free_scratch(M, s);
   CHECK(used == 0 && blocks.empty());
 }""".replace("FIRST", str(first)))
+
+
+@pytest.mark.parametrize("nf", [9000, 200_000, 700_000])
+def test_a_batch_that_fits_with_the_first_figures_runs(tmp_path, nf):
+    """Memory for the first figures per frame but not for the roomy ones: the batch gets the first,
+    keeps them on the next call, and a smaller batch, or a larger limit, gets the roomy ones."""
+    _run(tmp_path, r"""
+Scratch s;
+limit = (size_t)1 << 62;
+CHECK(ensure_scratch(M, s, NF, true) == M3E_OK && sound(s) && s.hits_cap > 128 * NF && s.trip_cap > 64 * NF);
+const size_t roomy = used;
+free_scratch(M, s);
+limit = roomy - 1;
+CHECK(ensure_scratch(M, s, NF, true) == M3E_OK && sound(s) && holds(s, NF));
+CHECK(s.hits_cap == 128 * NF && s.trip_cap == 64 * NF && s.combo_cap == 192 * NF);
+const size_t lean = used;
+const void* hf = s.hf;
+calls = 0;
+CHECK(ensure_scratch(M, s, NF, true) == M3E_OK && calls == 0 && s.hf == hf);
+CHECK(ensure_scratch(M, s, NF / 2, true) == M3E_OK && calls == 0 && s.hf == hf);
+free_scratch(M, s);
+limit = lean - 1;  // not even the first figures
+CHECK(ensure_scratch(M, s, NF, true) == M3E_ENOMEM && sound(s));
+CHECK(ensure_scratch(M, s, NF / 8, true) == M3E_OK && sound(s) && holds(s, NF / 8) && s.hits_cap >= 384 * (NF / 8));
+limit = 3 * roomy;
+CHECK(ensure_scratch(M, s, NF, true) == M3E_OK && sound(s) && s.hits_cap > 128 * NF);
+free_scratch(M, s);
+CHECK(used == 0);""".replace("NF", str(nf)))
