@@ -177,8 +177,13 @@ void make_devcfg(const m3e_config& c, DevCfg& d) {
   d.dr12 = (float)(c.r_mm[2] - c.r_mm[1]);
   d.zoff2 = (float)c.half_len_mm[2];
   d.izw2 = (float)(NZB / (2.0 * c.half_len_mm[2]));
-  d.c01 = (float)(std::cos(c.phi01_max) * c.r_mm[0] * c.r_mm[1]);
-  d.c12 = (float)(std::cos(c.phi12_max) * c.r_mm[1] * c.r_mm[2]);
+  // (an infinite cut has no cosine, and no pair passes it: a threshold of infinity says so to
+  // the comparison and to the sign of a difference alike, which a NaN does not)
+  const auto phi_threshold = [](double phi_max, double ra, double rb) {
+    return std::isinf(phi_max) ? INFINITY : (float)(std::cos(phi_max) * ra * rb);
+  };
+  d.c01 = phi_threshold(c.phi01_max, c.r_mm[0], c.r_mm[1]);
+  d.c12 = phi_threshold(c.phi12_max, c.r_mm[1], c.r_mm[2]);
   d.dl_max = (float)c.dlambda_max;
   d.rtc_lo2 = (float)(4.0 * c.rtc_min * c.rtc_min);
   d.rtc_hi2 = (float)(4.0 * c.rtc_max * c.rtc_max);
