@@ -66,6 +66,7 @@ int m3e::m3e_set_error(int code, const char* fmt, ...) {
 struct m3e_ctx {
   int device = 0;
   int sms = 1;
+  size_t smem_limit = 0;        // shared memory that a block may have
   int fused_bpsm = 1, group_bpsm = 1, s1_bpsm = 1, s2_bpsm = 1, s3_bpsm = 1, s4_bpsm = 1, s1c_bpsm = 1, s1m_bpsm = 1;
   int grab = 4;
   int defer_hits = W_HITS;
@@ -382,6 +383,7 @@ int m3e_create(const m3e_config* cfg, int cuda_device, m3e_ctx** out) {
     return fail(M3E_ECUDA, "cudaGetDeviceProperties");
   }
   x->sms = prop.multiProcessorCount;
+  x->smem_limit = prop.sharedMemPerBlockOptin;
   x->fused_bpsm = fused_blocks_per_sm();
   x->group_bpsm = group_blocks_per_sm();
   x->s1_bpsm = stage_blocks_per_sm(1);
@@ -706,7 +708,7 @@ extern "C" int m3e_ingest(m3e_ctx* x, const int32_t* d_hits, int64_t n_hits, flo
   if (!d_hits || !d_x || !d_y || !d_z) return fail(M3E_EINVAL, "NULL hit or coordinate array");
   DeviceGuard guard(x->device);
   CUDA_TRY(launch_ingest(x->dc, d_hits, n_hits, x->col_lut, x->row_lut, d_x, d_y, d_z, d_phi, x->err,
-                         x->sms, s));
+                         x->sms, x->smem_limit, s));
   x->last_launches = 1;
   return M3E_OK;
 }

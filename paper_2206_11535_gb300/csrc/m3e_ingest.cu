@@ -172,19 +172,21 @@ struct IngestCall {
   float *x, *y, *z, *phi;
   int* err;
   int sms;
+  size_t smem_limit;  // shared memory that a block may have
   cudaStream_t s;
 };
 
 template <bool VEC, bool PHI, bool HV>
 cudaError_t launch_ingest_t(const IngestCall& q) {
-  if (q.n <= INGEST_SMALL) {
+  const size_t sm = ingest_smem_bytes(q.c);
+  // a geometry whose tables do not fit an SM (up to 384 KB) never gets the copies
+  if (q.n <= INGEST_SMALL || sm > q.smem_limit) {
     const int64_t units = VEC ? (q.n + 3) / 4 : q.n;
     const int64_t want = (units + INGEST_SMALL_THREADS - 1) / INGEST_SMALL_THREADS, most = (int64_t)q.sms * 16;
     k_ingest_small<VEC, PHI, HV><<<(int)(want < most ? want : most), INGEST_SMALL_THREADS, 0, q.s>>>(
         q.c, q.hits, q.n, q.col_lut, q.row_lut, q.x, q.y, q.z, q.phi, q.err);
     return cudaGetLastError();
   }
-  const size_t sm = ingest_smem_bytes(q.c);
   cudaError_t e = cudaFuncSetAttribute(k_ingest<VEC, PHI, HV>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
   if (e != cudaSuccess) return e;
   k_ingest<VEC, PHI, HV><<<q.sms, INGEST_THREADS, sm, q.s>>>(q.c, q.hits, q.n, q.col_lut, q.row_lut, q.x, q.y, q.z,
@@ -195,9 +197,10 @@ cudaError_t launch_ingest_t(const IngestCall& q) {
 }  // namespace
 
 cudaError_t launch_ingest(const DevCfg& c, const int32_t* hits, int64_t n, const float4* col_lut, const float* row_lut,
-                          float* x, float* y, float* z, float* phi, int* err, int sms, cudaStream_t s) {
+                          float* x, float* y, float* z, float* phi, int* err, int sms, size_t smem_limit,
+                          cudaStream_t s) {
   auto al = [](const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; };  // NULL is aligned
-  const IngestCall q{c, hits, n, col_lut, row_lut, x, y, z, phi, err, sms, s};
+  const IngestCall q{c, hits, n, col_lut, row_lut, x, y, z, phi, err, sms, smem_limit, s};
   if (!(al(x) && al(y) && al(z) && al(phi)))
     return phi ? launch_ingest_t<false, true, false>(q) : launch_ingest_t<false, false, false>(q);
   if (al(hits)) return phi ? launch_ingest_t<true, true, true>(q) : launch_ingest_t<true, false, true>(q);

@@ -141,7 +141,8 @@ size_t cta_smem_bytes();
 
 // Hit ingest (m3e_ingest.cu): addresses -> FP32 x, y, z (and phi unless null) as SoA.
 cudaError_t launch_ingest(const DevCfg& c, const int32_t* hits, int64_t n, const float4* col_lut, const float* row_lut,
-                          float* x, float* y, float* z, float* phi, int* err, int sms, cudaStream_t s);
+                          float* x, float* y, float* z, float* phi, int* err, int sms, size_t smem_limit,
+                          cudaStream_t s);
 
 // Gradient of the fit chi2 (m3e_grad.cu).
 int fit_grad_blocks_per_sm(bool grad);
