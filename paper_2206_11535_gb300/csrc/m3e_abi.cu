@@ -773,6 +773,9 @@ extern "C" int m3e_select_frames_noalloc(m3e_ctx* x, const int32_t* d_hits, cons
   x->prof_valid = false;
   if (n_frames == 0) return M3E_OK;
   DeviceGuard guard(x->device);
+  int* scratch = nullptr;  // looked up by the first call, whatever its size: later ones may be captured
+  rc = noalloc_scratch(x->device, &scratch);
+  if (rc) return rc;
   if (n_frames <= SMALL_FRAMES) {  // no scratch at all
     KParams ps = base_params(x, x->main);
     ps.hits = d_hits;
@@ -784,9 +787,6 @@ extern "C" int m3e_select_frames_noalloc(m3e_ctx* x, const int32_t* d_hits, cons
     x->last_launches = 2;
     return M3E_OK;
   }
-  int* scratch = nullptr;
-  rc = noalloc_scratch(x->device, &scratch);
-  if (rc) return rc;
   KParams p{};
   p.col_lut = x->col_lut;
   p.row_lut = x->row_lut;
