@@ -512,14 +512,14 @@ def _fit_chi2_function():
 
     class FitChi2(torch.autograd.Function):
         """Sum of the track chi2 of frozen candidates as a function of the 25 alignment
-        and field-scale parameters.  One fit pass per step: when the parameters want a
-        gradient, m3e_fit_grad computes it with the sum and the 25 values are kept for the
+        and field-scale parameters.  One fit pass per step: when a gradient is wanted,
+        m3e_fit_grad computes it with the sum and the 25 values are kept for the
         backward (nothing per candidate is); else the sum alone."""
 
         @staticmethod
-        def forward(fctx, params, m3e_ctx, hits, off, cand):
+        def forward(fctx, params, m3e_ctx, hits, off, cand, want_grad):
             p = params.detach().to(torch.float32)
-            s, g = m3e_ctx.fit_grad(hits, off, cand, p, grad=fctx.needs_input_grad[0])
+            s, g = m3e_ctx.fit_grad(hits, off, cand, p, grad=want_grad)
             if g is not None:
                 fctx.save_for_backward(g)
             return s.to(params.dtype).reshape(())
@@ -527,7 +527,7 @@ def _fit_chi2_function():
         @staticmethod
         def backward(fctx, g_out):
             (g,) = fctx.saved_tensors
-            return (g_out * g).to(g_out.dtype), None, None, None, None
+            return (g_out * g).to(g_out.dtype), None, None, None, None, None
 
     return FitChi2
 
@@ -535,9 +535,16 @@ def _fit_chi2_function():
 _FIT = None
 
 
+def _grad_enabled() -> bool:
+    import torch
+    return torch.is_grad_enabled()
+
+
 def fit_chi2_sum(params, ctx: "Context", hits, off, cand):
     """Differentiable sum of the track chi2 (torch.autograd.Function over m3e_fit_grad)."""
     global _FIT
     if _FIT is None:
         _FIT = _fit_chi2_function()
-    return _FIT.apply(params, ctx, hits, off, cand)
+    # (within forward the grad mode is off, and a parameter that requires a gradient wants one
+    # also under no_grad)
+    return _FIT.apply(params, ctx, hits, off, cand, params.requires_grad and _grad_enabled())
