@@ -14,15 +14,28 @@
 // reverse sweep by hand, recomputing each triplet's intermediate values instead
 // of storing them.  d chi2 / d(field scale) = 2 chi2 / scale exactly: the scale
 // enters only through sigma_MS ~ 1/p and the two triplets' weights scale alike.
-// Sums: per-thread FP32 over its candidates, per-block FP64, then one block in a
-// fixed order (deterministic for a given grid).
+// Sums: per thread FP32 with its rounding errors kept beside it, per block FP64, then
+// one block in a fixed order (deterministic for a given grid).
 #include "m3e_device.cuh"
 
 namespace m3e {
 namespace {
 
 constexpr int GT = 128;            // threads per block
-constexpr int NG = 27;             // chi2, 24 alignment sums, chi2 of the finite gradients, valid candidates
+constexpr int NS = 26;             // chi2, 24 alignment sums, chi2 of the finite gradients
+constexpr int NG = NS + 1;         // and the number of valid candidates
+
+// A running sum and the sum of its rounding errors (Knuth's two-sum), so that the sum of a
+// thread's candidates is as good however many they are.  The gradient's 26 sums live in shared
+// memory: 971,437 candidates take 82 us (81 with plain sums in registers), 88 with 3 blocks per
+// SM instead of 4, 101 with both parts in registers.
+__device__ __forceinline__ void add_to(float2& s, float v) {
+  const float t = __fadd_rn(s.x, v), b = __fsub_rn(t, s.x);
+  s.y = __fadd_rn(s.y, __fadd_rn(__fsub_rn(s.x, __fsub_rn(t, b)), __fsub_rn(v, b)));
+  s.x = t;
+}
+// (a sum beyond FP32's range is infinite, as a plain one, and has no error)
+__device__ __forceinline__ float error_of(const float2& s) { return isfinite(s.x) ? s.y : 0.f; }
 
 struct AlignSm {
   float R[4][9];                   // rotation of each layer (row-major)
@@ -213,10 +226,12 @@ struct GradParams {
 };
 
 template <bool GRAD>
-__global__ void __launch_bounds__(GT) k_fit_grad(const __grid_constant__ DevCfg C, const __grid_constant__ GradParams G) {
+__global__ void __launch_bounds__(GT, GRAD ? 4 : 8)
+    k_fit_grad(const __grid_constant__ DevCfg C, const __grid_constant__ GradParams G) {
   __shared__ AlignSm A;
-  static_assert(NG % 2 == 1, "odd row stride and 8 words between the warps: no bank conflicts");
-  __shared__ __align__(8) float red[GRAD ? GT / 32 : 1][GRAD ? 32 * NG + 8 : 4 * (GT / 32)];
+  __shared__ float2 sums[GRAD ? NS : 1][GT];  // the threads' running sums
+  __shared__ double wsum[GT / 32];
+  __shared__ unsigned wvalid[GT / 32];
   pdl_trigger();
   if (threadIdx.x < 4) {
     const int L = threadIdx.x;
@@ -228,10 +243,16 @@ __global__ void __launch_bounds__(GT) k_fit_grad(const __grid_constant__ DevCfg 
   __syncthreads();
   const int64_t n_hits = G.off[G.n_frames];
   const float kB = C.kB * A.scale;
-  // chi2; per layer the gradient and its moment; chi2 of the candidates in the gradient; count
-  float acc[NG];
+  // chi2; per layer the gradient and its moment; chi2 of the candidates in the gradient
 #pragma unroll
-  for (int k = 0; k < NG; ++k) acc[k] = 0.f;
+  for (int k = 0; k < (GRAD ? NS : 0); ++k) sums[k][threadIdx.x] = make_float2(0.f, 0.f);
+  const auto add = [&](int k, float v) {
+    float2 s = sums[k][threadIdx.x];
+    add_to(s, v);
+    sums[k][threadIdx.x] = s;
+  };
+  float2 csum = make_float2(0.f, 0.f);
+  unsigned valid = 0;
   for (int64_t i = blockIdx.x * (int64_t)GT + threadIdx.x; i < G.n_cand; i += (int64_t)gridDim.x * GT) {
     const int4 q = __ldg(G.cand + i);
     const int qi[4] = {q.x, q.y, q.z, q.w};
@@ -328,59 +349,65 @@ __global__ void __launch_bounds__(GT) k_fit_grad(const __grid_constant__ DevCfg 
 #pragma unroll
             for (int L = 0; L < 4; ++L) {
               const float qx = P[L][0] - A.d[L][0], qy = P[L][1] - A.d[L][1], qz = P[L][2] - A.d[L][2];
-              acc[1 + 6 * L] += g[L][0];
-              acc[2 + 6 * L] += g[L][1];
-              acc[3 + 6 * L] += g[L][2];
-              acc[4 + 6 * L] += qy * g[L][2] - qz * g[L][1];
-              acc[5 + 6 * L] += qz * g[L][0] - qx * g[L][2];
-              acc[6 + 6 * L] += qx * g[L][1] - qy * g[L][0];
+              add(1 + 6 * L, g[L][0]);
+              add(2 + 6 * L, g[L][1]);
+              add(3 + 6 * L, g[L][2]);
+              add(4 + 6 * L, qy * g[L][2] - qz * g[L][1]);
+              add(5 + 6 * L, qz * g[L][0] - qx * g[L][2]);
+              add(6 + 6 * L, qx * g[L][1] - qy * g[L][0]);
             }
-            acc[25] += chi2;
+            add(25, chi2);
           }
         }
       }
     }
     if (ok) {
-      acc[0] += chi2;
-      acc[26] += 1.f;
+      add_to(csum, chi2);
+      ++valid;
     }
     if (G.chi2_each) G.chi2_each[i] = ok ? chi2 : __int_as_float(0x7fc00000);
     if (G.kappa_each) G.kappa_each[i] = ok ? kb_out : __int_as_float(0x7fc00000);
   }
   // block sums in FP64, fixed order
   const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
+  double v = 0.0;
   if (GRAD) {
-    // the threads' sums side by side in shared memory, then four threads per output, each
-    // adding 32 of them (8 times fewer FP64 additions, which are slow here, than a shuffle
-    // tree per output)
-#pragma unroll
-    for (int k = 0; k < NG; ++k) red[wp][lane * NG + k] = acc[k];
+    sums[0][threadIdx.x] = csum;
     __syncthreads();
+    // four threads per output, each adding 32 of the sums (8 times fewer FP64 additions, which
+    // are slow here, than a shuffle tree per output), from its own lane on: no bank conflicts
     const int k = threadIdx.x >> 2, part = threadIdx.x & 3;
-    double v = 0.0;
-    if (k < NG) {
+    float e = 0.f;
+    if (k < NS) {
 #pragma unroll 8
-      for (int j = 0; j < 32; ++j) v += (double)red[part][j * NG + k];
+      for (int j = 0; j < 32; ++j) {
+        const float2 q = sums[k][32 * part + ((j + lane) & 31)];
+        v += (double)q.x;
+        e += error_of(q);
+      }
     }
+    v += (double)e;
     v += __shfl_xor_sync(FULL, v, 1);
     v += __shfl_xor_sync(FULL, v, 2);
-    if (k < NG && part == 0) G.partial[(int64_t)k * gridDim.x + blockIdx.x] = v;
+    if (k < NS && part == 0) G.partial[(int64_t)k * gridDim.x + blockIdx.x] = v;
   } else {
-    double* const dred = reinterpret_cast<double*>(&red[0][0]);
-    double v = acc[0];
+    v = (double)csum.x + (double)error_of(csum);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(FULL, v, o);
-    const unsigned nv = __reduce_add_sync(FULL, (unsigned)acc[26]);
-    if (lane == 0) {
-      dred[wp] = v;
-      dred[GT / 32 + wp] = (double)nv;
-    }
-    __syncthreads();
-    if (threadIdx.x < 2) {
-      double t = 0.0;
-      for (int k = 0; k < GT / 32; ++k) t += dred[threadIdx.x * (GT / 32) + k];
-      G.partial[(int64_t)(threadIdx.x ? 26 : 0) * gridDim.x + blockIdx.x] = t;
-    }
+    if (lane == 0) wsum[wp] = v;
+  }
+  valid = __reduce_add_sync(FULL, valid);
+  if (lane == 0) wvalid[wp] = valid;
+  __syncthreads();
+  if (threadIdx.x == 32) {
+    unsigned n = 0;
+    for (int k = 0; k < GT / 32; ++k) n += wvalid[k];
+    G.partial[(int64_t)NS * gridDim.x + blockIdx.x] = (double)n;
+  }
+  if (!GRAD && threadIdx.x == 0) {
+    v = 0.0;
+    for (int k = 0; k < GT / 32; ++k) v += wsum[k];
+    G.partial[blockIdx.x] = v;
   }
 }
 
@@ -391,7 +418,7 @@ __global__ void __launch_bounds__(32 * NG)
                  unsigned long long* n_valid, float* chi2_sum, float* grad) {
   __shared__ double sum[NG];
   // without the gradient two warps: the sum and the count
-  const int k = grad ? threadIdx.x >> 5 : (threadIdx.x >> 5) * (NG - 1), lane = threadIdx.x & 31;
+  const int k = grad ? threadIdx.x >> 5 : (threadIdx.x >> 5) * NS, lane = threadIdx.x & 31;
   pdl_wait();
   double v = 0.0;
 #pragma unroll 16
@@ -401,7 +428,7 @@ __global__ void __launch_bounds__(32 * NG)
   if (lane == 0) sum[k] = v;
   __syncthreads();
   const int t = threadIdx.x;
-  if (t == 31) *n_valid = (unsigned long long)sum[26];
+  if (t == 31) *n_valid = (unsigned long long)sum[NS];
   if (t == 0 && chi2_sum) *chi2_sum = (float)sum[0];
   if (!grad) return;
   if (t == 32) grad[24] = (float)(2.0 * sum[25] / (double)params[24]);
