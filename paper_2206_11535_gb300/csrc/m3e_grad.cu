@@ -431,7 +431,8 @@ __global__ void __launch_bounds__(32 * NG)
   if (t == 31) *n_valid = (unsigned long long)sum[NS];
   if (t == 0 && chi2_sum) *chi2_sum = (float)sum[0];
   if (!grad) return;
-  if (t == 32) grad[24] = (float)(2.0 * sum[25] / (double)params[24]);
+  // (no candidate is valid at a scale of 0, and the gradient of the empty sum is 0)
+  if (t == 32) grad[24] = sum[25] != 0.0 ? (float)(2.0 * sum[25] / (double)params[24]) : 0.f;
   if (t >= 64 && t < 76) {
     const int L = (t - 64) / 3, r = (t - 64) % 3;
     grad[6 * L + r] = (float)sum[1 + 6 * L + r];
