@@ -204,8 +204,11 @@ int m3e_select_frames_host(m3e_ctx* ctx, const int32_t* h_hits, const int64_t* h
  * address or frame size (and clear the latch), else M3E_OK. */
 int m3e_check(m3e_ctx* ctx, cudaStream_t stream);
 
-/* Tuning of the persistent kernel: frames taken per work-queue grab (1..64) and
- * resident CTAs per SM (0 = as many as fit). */
+/* Tuning of the persistent kernels.  frames_per_grab (1..64): frames that a warp takes
+ * from the work queue at a time, at most; a batch gives every resident warp at least
+ * two grabs, and m3e_select_frames_noalloc always takes eight frames per CTA.
+ * ctas_per_sm: resident CTAs per SM of m3e_select_frames_fused and, up to the four
+ * that fit, of m3e_select_frames_noalloc (0 = as many as fit). */
 int m3e_set_launch(m3e_ctx* ctx, int frames_per_grab, int ctas_per_sm);
 
 /* Size the context's scratch for batches of up to max_frames frames, so that the

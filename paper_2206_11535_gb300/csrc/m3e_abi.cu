@@ -67,7 +67,7 @@ struct m3e_ctx {
   int device = 0;
   int sms = 1;
   size_t smem_limit = 0;        // shared memory that a block may have
-  int fused_bpsm = 1, group_bpsm = 1, s1_bpsm = 1, s2_bpsm = 1, s3_bpsm = 1, s4_bpsm = 1, s1c_bpsm = 1, s1m_bpsm = 1;
+  int fused_bpsm = 1, group_bpsm = 1, noalloc_bpsm = 1, s1_bpsm = 1, s2_bpsm = 1, s3_bpsm = 1, s4_bpsm = 1, s1c_bpsm = 1, s1m_bpsm = 1;
   int grab = 4;
   int defer_hits = W_HITS;
   int mid_threads = CTA_THREADS;  // threads of a stage-1 middle-tier CTA
@@ -298,9 +298,9 @@ Route route_of(int form, int64_t n, bool debug, bool timed, const void* stats) {
 }
 
 // One decision-only batch in the group form: p.work and the deferred list are its only scratch.
-int enqueue_group(m3e_ctx* x, const KParams& p, cudaStream_t s) {
+int enqueue_group(m3e_ctx* x, const KParams& p, int bpsm, cudaStream_t s) {
   CUDA_TRY(cudaMemsetAsync(p.work, 0, 2 * sizeof(int), s));  // queue head and deferred count
-  CUDA_TRY(launch_group(x->dc, p, x->sms * x->group_bpsm, s));
+  CUDA_TRY(launch_group(x->dc, p, x->sms * bpsm, s));
   CUDA_TRY(launch_deferred(x->dc, p, 2 * x->sms, false, s, true));
   x->last_launches = 2;
   return M3E_OK;
@@ -317,7 +317,7 @@ int enqueue(m3e_ctx* x, Scratch& sc, KParams p, int form, bool debug, cudaStream
     x->last_launches = 2;
     return M3E_OK;
   }
-  if (route == ROUTE_GROUP) return enqueue_group(x, p, s);
+  if (route == ROUTE_GROUP) return enqueue_group(x, p, x->group_bpsm, s);
   // frames per queue grab: at least two grabs for every resident warp, so that a batch of
   // a few frames per warp spreads over all of them
   const int64_t warps = (int64_t)x->sms * WARPS_PER_CTA * (form == FORM_FUSED ? x->fused_bpsm : x->s1_bpsm);
@@ -385,7 +385,7 @@ int m3e_create(const m3e_config* cfg, int cuda_device, m3e_ctx** out) {
   x->sms = prop.multiProcessorCount;
   x->smem_limit = prop.sharedMemPerBlockOptin;
   x->fused_bpsm = fused_blocks_per_sm();
-  x->group_bpsm = group_blocks_per_sm();
+  x->group_bpsm = x->noalloc_bpsm = group_blocks_per_sm();
   x->s1_bpsm = stage_blocks_per_sm(1);
   x->s2_bpsm = stage_blocks_per_sm(2);
   x->s3_bpsm = stage_blocks_per_sm(3);
@@ -467,6 +467,7 @@ int m3e_set_launch(m3e_ctx* x, int frames_per_grab, int ctas_per_sm) {
   if (ctas_per_sm < 0 || ctas_per_sm > maxb) return fail(M3E_EINVAL, "ctas_per_sm 0..%d", maxb);
   x->grab = frames_per_grab;
   x->fused_bpsm = ctas_per_sm ? ctas_per_sm : maxb;
+  x->noalloc_bpsm = ctas_per_sm ? std::min(ctas_per_sm, x->group_bpsm) : x->group_bpsm;
   return M3E_OK;
 }
 
@@ -803,7 +804,7 @@ extern "C" int m3e_select_frames_noalloc(m3e_ctx* x, const int32_t* d_hits, cons
   p.n_frames = n_frames;
   p.keep = d_keep;
   p.reason = d_reason;
-  return enqueue_group(x, p, s);
+  return enqueue_group(x, p, x->noalloc_bpsm, s);
 }
 
 // ------------------------------------------------------------------ persistent batched form
