@@ -245,8 +245,9 @@ typedef struct {
 
 /* Time the staged form on a calibration batch (device buffers as for
  * m3e_select_frames) over launch parameters and keep the fastest in the
- * context: a grid of frames_per_grab (1..16) x defer_hits (96, 128, 160) x
- * stage-1 CTAs per SM (all, half), then, one axis at a time from that point, the
+ * context: a grid of frames_per_grab (the current setting and those of 1..16 that
+ * the batch is large enough to run with) x defer_hits (96, 128, 160) x stage-1
+ * CTAs per SM (all, half), then, one axis at a time from that point, the
  * middle tier's CTA size (128, 256, 512 threads) and the track stage's CTAs per
  * SM.  Synchronises the context's device; decisions do not depend on the
  * parameters.  Each configuration is timed as the median of five runs after a

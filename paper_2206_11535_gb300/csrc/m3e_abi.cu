@@ -306,6 +306,14 @@ int enqueue_group(m3e_ctx* x, const KParams& p, int bpsm, cudaStream_t s) {
   return M3E_OK;
 }
 
+// Frames per queue grab of a batch of n frames, of `grab` at most: at least two grabs for
+// every resident warp (bpsm CTAs per SM), so that a batch of a few frames per warp spreads
+// over all of them.
+int grab_of(const m3e_ctx* x, int64_t n, int grab, int bpsm) {
+  const int64_t warps = (int64_t)x->sms * WARPS_PER_CTA * bpsm;
+  return (int)std::max<int64_t>(1, std::min<int64_t>(grab, n / (2 * warps)));
+}
+
 // Enqueue one batch on stream s: form 0 staged (5 kernels; smaller batches as route_of says
 // unless `reroute` is false), 1 fused warp kernel, 2 plain CTA-per-frame kernel; forms 0 and
 // 1 finish with the deferred-frame kernel.  Timing events are recorded when `timed`.
@@ -318,10 +326,7 @@ int enqueue(m3e_ctx* x, Scratch& sc, KParams p, int form, bool debug, cudaStream
     return M3E_OK;
   }
   if (route == ROUTE_GROUP) return enqueue_group(x, p, x->group_bpsm, s);
-  // frames per queue grab: at least two grabs for every resident warp, so that a batch of
-  // a few frames per warp spreads over all of them
-  const int64_t warps = (int64_t)x->sms * WARPS_PER_CTA * (form == FORM_FUSED ? x->fused_bpsm : x->s1_bpsm);
-  p.grab = (int)std::max<int64_t>(1, std::min<int64_t>(p.grab, p.n_frames / (2 * warps)));
+  p.grab = grab_of(x, p.n_frames, p.grab, form == FORM_FUSED ? x->fused_bpsm : x->s1_bpsm);
   if (form == FORM_PLAIN) {
     if (timed) CUDA_TRY(cudaEventRecord(x->pe[0], s));
     CUDA_TRY(launch_plain(x->dc, p, debug, s));
@@ -904,10 +909,19 @@ extern "C" int m3e_autotune(m3e_ctx* x, const int32_t* d_hits, const int64_t* d_
   CUDA_TRY(cudaEventCreate(&e1));
   constexpr float AUTOTUNE_MARGIN = 0.02f;
   const int s1max = stage_blocks_per_sm(1);
-  const int grabs[] = {1, 2, 4, 8, 16};
   const int dhits[] = {96, 128, W_HITS};
   const int s1s[] = {s1max, s1max > 2 ? (s1max + 1) / 2 : s1max};
   const int g0 = x->grab, d0 = x->defer_hits, b0 = x->s1_bpsm;
+  // frames per grab: the current setting, then every other number that this batch really runs
+  // with (grab_of), each once; a setting that never ran is not put in force
+  const auto grabs = [&](int b) {
+    std::vector<int> v = {g0};
+    for (int g : {1, 2, 4, 8, 16}) {
+      const int e = grab_of(x, n, g, b);
+      if (std::none_of(v.begin(), v.end(), [&](int w) { return grab_of(x, n, w, b) == e; })) v.push_back(e);
+    }
+    return v;
+  };
   auto run = [&](float* ms) -> int {
     KParams p = base_params(x, x->main);
     p.hits = d_hits;
@@ -933,9 +947,9 @@ extern "C" int m3e_autotune(m3e_ctx* x, const int32_t* d_hits, const int64_t* d_
   rc = run(&ms_def);
   float best = ms_def;
   int bg = g0, bd = d0, bb = b0, tried = 1;
-  for (int g : grabs)
-    for (int d : dhits)
-      for (int b : s1s) {
+  for (int b : s1s)
+    for (int g : grabs(b))
+      for (int d : dhits) {
         if (rc) break;
         x->grab = g;
         x->defer_hits = d;
