@@ -306,8 +306,8 @@ int m3e_ingest(m3e_ctx* ctx, const int32_t* d_hits, int64_t n_hits, float* d_x, 
  *     make that first call before any stream capture.  The address is cached per
  *     device; m3e_create clears the cache, so after a cudaDeviceReset create a
  *     new context before calling again.
- *   - Frames above the context's warp-tier size (set by m3e_autotune) go to
- *     CTA-per-frame kernels.
+ *   - Frames of more than 160 hits (512 in a call of at most 2048 frames) go to a
+ *     CTA-per-frame kernel, whatever m3e_autotune chose for the staged form.
  *   - The array is shared by all calls on a device and keeps the last call's
  *     contents; the call clears what must start at zero.  Calls that overlap on
  *     the GPU (other streams, other contexts of the same device, other threads)

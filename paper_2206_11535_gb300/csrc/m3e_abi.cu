@@ -298,7 +298,10 @@ Route route_of(int form, int64_t n, bool debug, bool timed, const void* stats) {
 }
 
 // One decision-only batch in the group form: p.work and the deferred list are its only scratch.
-int enqueue_group(m3e_ctx* x, const KParams& p, int bpsm, cudaStream_t s) {
+// It defers by its own stage's size, not by the tuned one: that is measured on the staged form,
+// where a deferred frame goes to a middle tier, and here it goes to the largest stage.
+int enqueue_group(m3e_ctx* x, KParams p, int bpsm, cudaStream_t s) {
+  p.defer_hits = W_HITS;
   CUDA_TRY(cudaMemsetAsync(p.work, 0, 2 * sizeof(int), s));  // queue head and deferred count
   CUDA_TRY(launch_group(x->dc, p, x->sms * bpsm, s));
   CUDA_TRY(launch_deferred(x->dc, p, 2 * x->sms, false, s, true));
@@ -802,7 +805,6 @@ extern "C" int m3e_select_frames_noalloc(m3e_ctx* x, const int32_t* d_hits, cons
   p.defer_count = scratch + 1;
   p.in_list = scratch + NOALLOC_HEAD;
   p.in_count = scratch + 1;
-  p.defer_hits = x->defer_hits;  // the same warp/CTA split as the fused entry point
   p.grab = x->grab;
   p.hits = d_hits;
   p.off = d_frame_off;
