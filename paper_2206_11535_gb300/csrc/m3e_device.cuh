@@ -1153,8 +1153,8 @@ __device__ __forceinline__ void bucket_scan(const G& g, S& sm) {
 
 // Which of n <= 32 hits (xs, ys: 16-byte aligned, readable to the next multiple of four)
 // pass the Phi cut with the hit whose coordinates xx, yy hold twice: bit q for hit q.  The
-// test is phi_pass, two hits per instruction; the sign of (product - c), which is exact, is
-// shifted into the mask, the last hit first.
+// test is phi_pass, two hits per instruction; the sign of (product - c), which its rounding
+// leaves as it is, is shifted into the mask, the last hit first.
 __device__ __forceinline__ uint32_t phi_mask(const float* xs, const float* ys, int n, unsigned long long xx,
                                              unsigned long long yy, float c) {
   const unsigned long long mc = pack2(-c, -c);
@@ -1183,8 +1183,8 @@ __device__ __forceinline__ uint32_t phi_mask(const float* xs, const float* ys, i
 //      those hits that all lanes take together (one broadcast load per hit);
 //   2. the pairs of layer-1 hits that have Phi12 partners, numbered by a prefix sum
 //      and listed with their layer-0 hit;
-//   3. the pairs, 32 at a time: each lane finds its pair's layer-1 hit (a search
-//      over the lanes' prefix), forms the z window (widened by 1e-3 mm against
+//   3. the pairs, 32 at a time: each lane takes its pair's layer-1 hit from the lane
+//      that the list names, forms the z window (widened by 1e-3 mm against
 //      rounding) and its bin range, and keeps the Phi12 partners inside it: the
 //      candidate triplets, numbered by a prefix sum and listed;
 //   4. the candidates, 32 at a time, through the exact Delta lambda and r_tc tests,

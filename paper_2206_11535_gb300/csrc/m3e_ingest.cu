@@ -21,7 +21,7 @@ namespace {
 constexpr int INGEST_THREADS = 1024;
 // Steps in flight per thread: the output streams of a step lie a grid's width apart, and the
 // fewer of them are open the better DRAM takes them (85.5 M hits: 1 step 295 us, 2 steps 277,
-// 4 steps 300, 6 steps 298; 91% of the measured copy rate with 2).
+// 4 steps 300, 6 steps 298; in the benchmark 271 us, 93% of the measured copy rate).
 constexpr int INGEST_UNROLL = 2;
 constexpr int INGEST_SMALL_THREADS = 128;
 // Up to this many hits without the shared-memory tables, whose copies cost every CTA 183 KB:
