@@ -13,8 +13,9 @@
 // so that the chi2 equals the selection's at nominal alignment), then the
 // reverse sweep by hand, recomputing each triplet's intermediate values instead
 // of storing them, but for the arc angles and the small polar offset, which it takes
-// from the forward fit (the only transcendental functions).  d chi2 / d(field scale) = 2 chi2 / scale exactly: the scale
-// enters only through sigma_MS ~ 1/p and the two triplets' weights scale alike.
+// from the forward fit (the only transcendental functions).  d chi2 / d(field scale) =
+// 2 chi2 / scale exactly: the scale enters only through sigma_MS ~ 1/p and the two
+// triplets' weights scale alike.
 // Sums: per thread FP32 with its rounding errors kept beside it, per block FP64, then
 // one block in a fixed order (deterministic for a given grid).
 #include "m3e_device.cuh"

@@ -301,7 +301,7 @@ __device__ __forceinline__ void load_circle(const float4* __restrict__ rec, int6
 // tracks of the next frame are fetched into L1 while one is tested, and the combinations of all of
 // them are written behind one allocation, a fourth of the atomics on the one counter.
 // Bound by issue (849 warp instructions per throughput frame, 71% issue active, 10 CTAs per
-// SM at 48 registers; 9 CTAs at 56 take 2% longer, 12 CTAs 13%: 1e6 throughput frames 854 -> 719 us,
+// SM at 48 registers; 9 CTAs at 56 take 2% longer, 12 CTAs 13%): 1e6 throughput frames 854 -> 719 us,
 // 200,000 uneven frames 541 -> 283 us, most of that from frames that stop at the combination
 // cap.  Taking 16 frames at a time cost 745 and 535 us (heavy frames queue in one warp).
 // Before they are written the combinations go through the vertex's first two steps, which
