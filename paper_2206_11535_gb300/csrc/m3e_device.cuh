@@ -834,7 +834,7 @@ __device__ __forceinline__ void vertex_soft(const TrackR& A, const TrackR& B, co
 // roundings of the vertex depend on the order, and the numbers of the tracks depend on the form
 // and, where the threads of a CTA number them by arrival, on the run: with an order by value
 // every form and every run takes the same decision, whatever the order of a frame's hits.  (With
-// equal centres the circles do not meet, either way.)  1e6 throughput frames 5282 -> 5295 us.
+// equal centres the circles do not meet, either way.)  1e6 throughput frames 5264 -> 5283 us.
 __device__ __forceinline__ bool swapped(float acx, float acy, float bcx, float bcy) {
   return acx != bcx ? acx > bcx : acy > bcy;
 }

@@ -161,7 +161,7 @@ __device__ bool gate_wait(const KParams& P, int k) {
 // GATED (host entry point): the hits arrive while the kernel runs; a frame is
 // taken only after its chunk's arrival flag, and the hits are read past L1.
 // NOST: the instance for runs without statistics (no statistics code at all).
-// Bound by instruction issue and shared-memory latency (1,854 warp instructions per
+// Bound by instruction issue and shared-memory latency (1,857 warp instructions per
 // throughput frame at 66% issue active; shared-memory loads are the largest stall): 1e6
 // throughput frames 2.36 -> 2.15 ms with the packed partner masks, one decode per hit and no
 // address list, at 64 registers and 8 CTAs per SM (2.20 ms at 56 registers and 9 CTAs),
@@ -300,7 +300,7 @@ __device__ __forceinline__ void load_circle(const float4* __restrict__ rec, int6
 // A warp takes P.grab frames at a time: their states are read together, a lane each, the
 // tracks of the next frame are fetched into L1 while one is tested, and the combinations of all of
 // them are written behind one allocation, a fourth of the atomics on the one counter.
-// Bound by issue (849 warp instructions per throughput frame, 71% issue active, 10 CTAs per
+// Bound by issue (850 warp instructions per throughput frame, 71% issue active, 10 CTAs per
 // SM at 48 registers; 9 CTAs at 56 take 2% longer, 12 CTAs 13%): 1e6 throughput frames 854 -> 719 us,
 // 200,000 uneven frames 541 -> 283 us, most of that from frames that stop at the combination
 // cap.  Taking 16 frames at a time cost 745 and 535 us (heavy frames queue in one warp).
@@ -308,7 +308,7 @@ __device__ __forceinline__ void load_circle(const float4* __restrict__ rec, int6
 // three in four do not survive: their gathers of track circles from DRAM bounded stage 4 and
 // fit beside the arithmetic here (this stage 719 -> 817 us, stage 4 399 -> 225 us).  The next
 // frame's tracks went into four registers at first, and the kernel spilled 148 bytes a thread;
-// fetched into L1 instead, 44 bytes and 793 us.
+// fetched into L1 instead, nothing and 793 us.
 template <bool DEBUG, bool NOST = false>
 __global__ void __launch_bounds__(S3_WARPS * 32, 10)
     k_stage3(const __grid_constant__ DevCfg C, const __grid_constant__ KParams P, const __grid_constant__ SParams S) {
@@ -494,6 +494,7 @@ __global__ void __launch_bounds__(S3_WARPS * 32, 10)
 // Bound by the latency of the track records and by spills: 1e6 throughput frames 229 us at 64
 // registers (8 CTAs per SM) with every combination filtered again, 217 without that, 213 at 80
 // registers, 191 at 96, 200 at 128 (no spills, 4 CTAs per SM); 200,000 uneven frames 68 -> 59.
+// 205 with the e+ tracks ordered by value (vertex), which waits for both tracks' circles.
 constexpr int S4_WARPS = 4;
 
 template <bool DEBUG>
